@@ -87,7 +87,7 @@ __global__ void norm2_kernel(long long N, int n, const void *v, Reduce red) {
         Spinor<P>::load(v, N, e, a);
         T s = 0;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) s += a[k].re * a[k].re + a[k].im * a[k].im;
+        for (int k = 0; k < 12; ++k) s = fma(a[k].re, a[k].re, fma(a[k].im, a[k].im, s));
         acc.add(0, 0, s);
     }
     grid_reduce(red, acc, n);
@@ -106,9 +106,9 @@ __global__ void dot_norm_kernel(long long N, int n, const void *av, const void *
         T s0 = 0, s1 = 0, s2 = 0;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            s0 += a[k].re * b[k].re + a[k].im * b[k].im;
-            s1 += a[k].re * b[k].im - a[k].im * b[k].re;
-            s2 += b[k].re * b[k].re + b[k].im * b[k].im;
+            s0 = fma(a[k].re, b[k].re, fma(a[k].im, b[k].im, s0));
+            s1 = fma(a[k].re, b[k].im, fma(-a[k].im, b[k].re, s1));
+            s2 = fma(b[k].re, b[k].re, fma(b[k].im, b[k].im, s2));
         }
         acc.add(0, 0, s0);
         acc.add(1, 0, s1);
@@ -123,6 +123,7 @@ __global__ void cg_update_kernel(long long N, int n, void *x, void *r, const voi
                                  const SolverState *st) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
+    if (all_frozen(st, n)) return;
     RedAcc<1> acc;
     red_init(acc);
     ELEM_LOOP(N) {
@@ -142,7 +143,7 @@ __global__ void cg_update_kernel(long long N, int n, void *x, void *r, const voi
             xv[k].im = fma((TX)alpha, (TX)pv[k].im, xv[k].im);
             rv[k].re = fma(-alpha, qv[k].re, rv[k].re);
             rv[k].im = fma(-alpha, qv[k].im, rv[k].im);
-            s += rv[k].re * rv[k].re + rv[k].im * rv[k].im;
+            s = fma(rv[k].re, rv[k].re, fma(rv[k].im, rv[k].im, s));
         }
         Spinor<PX>::store(x, N, e, xv);
         Spinor<P>::store(r, N, e, rv);
@@ -311,6 +312,7 @@ __global__ void bicg_update_kernel(long long N, int n, void *x, void *r, const v
                                    const void *t, const void *rhat, Reduce red, const SolverState *st) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
+    if (all_frozen(st, n)) return;
     RedAcc<3> acc;
     red_init(acc);
     ELEM_LOOP(N) {
@@ -331,9 +333,9 @@ __global__ void bicg_update_kernel(long long N, int n, void *x, void *r, const v
             xv[k] = {xv[k].re + (TX)dx.re, xv[k].im + (TX)dx.im};
             cx<T> rn = csub(sv[k], cmulc(omega, tv[k]));
             sv[k] = rn;
-            s0 += hv[k].re * rn.re + hv[k].im * rn.im;
-            s1 += hv[k].re * rn.im - hv[k].im * rn.re;
-            s2 += rn.re * rn.re + rn.im * rn.im;
+            s0 = fma(hv[k].re, rn.re, fma(hv[k].im, rn.im, s0));
+            s1 = fma(hv[k].re, rn.im, fma(-hv[k].im, rn.re, s1));
+            s2 = fma(rn.re, rn.re, fma(rn.im, rn.im, s2));
         }
         Spinor<PX>::store(x, N, e, xv);
         Spinor<P>::store(r, N, e, sv);

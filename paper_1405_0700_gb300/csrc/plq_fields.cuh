@@ -400,117 +400,127 @@ __device__ __forceinline__ V warp_sum(V x, int lane, int active) {
 
 // Combine the accumulators of the whole grid (ncols right-hand-side columns
 // of RT right-hand sides each): within a warp the lanes of each column are
-// folded onto its first lanes, row after row; the warps of a block then add
-// their column sums into shared slots one warp after the other; each block
-// writes its partial sums to red.partials, and the last block to finish
-// (ticket counter) adds them in block order, stores the totals in
-// red.sums[k*n + r] and applies the finalize step to red.st[r].  Every thread
-// of every block must call it.
+// folded onto its first lanes; the warps' column sums are added in warp order,
+// kRedWarps warps per block barrier; each block writes its partial sums to
+// red.partials, and the last block to finish (ticket counter) adds them, every
+// thread striding over the blocks, stores the totals in red.sums[k*n + r] and
+// applies the finalize step to red.st[r].  The order is fixed for a launch
+// configuration.  Every thread of every block must call it.
+//
+// This tail is latency, not bandwidth: what counts is the chain of barriers,
+// fences and L2 round trips behind the last site.  So one thread fences for
+// its block (the barrier before it orders the other threads' stores), the
+// partial sums of a slot lie side by side (the last block reads 256 blocks in
+// one coalesced load per slot), and all loads of a slot group are in flight
+// together.  Measured as launches with no element to work on (all right-hand
+// sides frozen, 24^3x48): see grid_reduce figures at all_frozen().
+constexpr int kRedWarps = 8;
+
 template <int NV, int RT>
 __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int ncols) {
+    constexpr int W = NV * RT;                      // values per thread
+    constexpr int kCols = W > 4 ? 1 : PLQ_MAX_RHS;  // columns that fit wv (the wide forms have one)
+    __shared__ double wv[kRedWarps * kCols * W];    // (warp of the round, lane, value), later (warp, slot)
     __shared__ double slot[kPartialSlots];
-    __shared__ double tots[kPartialSlots];
     __shared__ bool last;
     const int tid = ltid(), lane = tid & 31, warp = tid >> 5, nthr = lsize(), nw = (nthr + 31) >> 5;
     const int active = min(32, nthr - warp * 32);  // lanes present in this thread's warp
     const int n = ncols * RT, slots = NV * n;
-    double *mine = red.partials + (size_t)blockIdx.x * kPartialSlots;
-    for (int t = tid; t < slots; t += nthr) slot[t] = 0.0;
-    double w[NV][RT];
+    double w[W];
 #pragma unroll
     for (int k = 0; k < NV; ++k)
 #pragma unroll
-        for (int t = 0; t < RT; ++t) w[k][t] = acc.v[k][t];
+        for (int t = 0; t < RT; ++t) w[k * RT + t] = acc.v[k][t];
     if (ncols == 1) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-            for (int t = 0; t < RT; ++t) w[k][t] = warp_sum(w[k][t], lane, active);
+        for (int k = 0; k < W; ++k) w[k] = warp_sum(w[k], lane, active);
     } else {
         const unsigned mask = active >= 32 ? 0xffffffffu : ((1u << active) - 1u);
         for (int o = ncols; o < 32; o += ncols) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k)
-#pragma unroll
-                for (int t = 0; t < RT; ++t) {
-                    const double y = __shfl_down_sync(mask, w[k][t], o);
-                    if (lane < ncols && lane + o < active) w[k][t] += y;
-                }
+            for (int k = 0; k < W; ++k) {
+                const double y = __shfl_down_sync(mask, w[k], o);
+                if (lane < ncols && lane + o < active) w[k] += y;
+            }
         }
     }
-    __syncthreads();
-    const int lead = min(ncols, active);  // lanes holding their warp's column sums
-    for (int ww = 0; ww < nw; ++ww) {
-        if (warp == ww && lane < lead) {
-            const int c = tid % ncols;
+    for (int t = tid; t < slots; t += nthr) slot[t] = 0.0;
+    for (int w0 = 0; w0 < nw; w0 += kRedWarps) {
+        if (w0 > 0) __syncthreads();
+        if (warp >= w0 && warp < w0 + kRedWarps && lane < min(ncols, active)) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k)
-#pragma unroll
-                for (int t = 0; t < RT; ++t) slot[k * n + c * RT + t] += w[k][t];
+            for (int k = 0; k < W; ++k) wv[((warp - w0) * ncols + lane) * W + k] = w[k];
         }
         __syncthreads();
+        const int w1 = min(nw, w0 + kRedWarps);
+        for (int t = tid; t < slots; t += nthr) {  // (a slot stays with its thread)
+            const int k = t / n, c = (t - k * n) / RT, v = k * RT + (t - k * n) - c * RT;
+            double s = slot[t];
+            for (int ww = w0; ww < w1; ++ww) {
+                int l = c - (32 * ww) % ncols;  // the lane of warp ww that holds column c
+                if (l < 0) l += ncols;
+                if (l < nthr - 32 * ww) s += wv[((ww - w0) * ncols + l) * W + v];
+            }
+            slot[t] = s;
+            if (w1 == nw) red.partials[(size_t)t * kMaxReduceBlocks + blockIdx.x] = s;
+        }
     }
-    for (int t = tid; t < slots; t += nthr) mine[t] = slot[t];
-    __threadfence();
     __syncthreads();
-    if (tid == 0) last = (atomicAdd(red.ticket, 1u) == gridDim.x - 1);
+    if (tid == 0) {
+        __threadfence();
+        last = (atomicAdd(red.ticket, 1u) == gridDim.x - 1);
+        if (last) __threadfence();
+    }
     __syncthreads();
     if (!last) return;
-    __threadfence();
-    // The last block sums every slot over the blocks in a fixed order.  With at
-    // least twice as many full warps as slots, g = (full warps) / slots warps
-    // share a slot: warp q of the slot's group takes blocks q*32 + lane,
-    // q*32 + lane + g*32, ... (four loads in flight per lane), then the group's
-    // warp sums are added in warp order.  Otherwise each warp takes whole slots,
-    // a partial last warp striding by its `active` lanes, so that every block is
-    // still visited.
-    const double *part = red.partials;
-    auto strided_sum = [&](int t, int first, int step) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int b = first;
-        for (; b + 3 * step < (int)gridDim.x; b += 4 * step) {
-            s0 += __ldcg(part + (size_t)b * kPartialSlots + t);
-            s1 += __ldcg(part + (size_t)(b + step) * kPartialSlots + t);
-            s2 += __ldcg(part + (size_t)(b + 2 * step) * kPartialSlots + t);
-            s3 += __ldcg(part + (size_t)(b + 3 * step) * kPartialSlots + t);
-        }
-        for (; b < (int)gridDim.x; b += step) s0 += __ldcg(part + (size_t)b * kPartialSlots + t);
-        return (s0 + s1) + (s2 + s3);
-    };
-    const int nfull = nthr >> 5;
-    const int g = nfull >= 2 * slots ? nfull / slots : 1;
-    if (g > 1) {
-        const int t = warp / g, q = warp % g;
-        if (warp < slots * g) {  // full warps only: slots * g <= nfull
-            double s = strided_sum(t, q * 32 + lane, g * 32);
-            s = warp_sum(s, lane, active);
-            if (lane == 0) slot[t * g + q] = s;  // slot[] is free again
-        }
-        __syncthreads();
-        if (tid < slots) {
-            double s = 0.0;
-            for (int k = 0; k < g; ++k) s += slot[tid * g + k];
-            tots[tid] = s;
-        }
-    } else {
-        for (int t = warp; t < slots; t += nw) {
-            double s = strided_sum(t, lane, active);
-            s = warp_sum(s, lane, active);
-            if (lane == 0) tots[t] = s;
+    // The last block: its first kRedWarps warps stride over the blocks, four
+    // slots at a time, then the warps' sums are added in warp order.
+    const int part = min(nthr, 32 * kRedWarps), pw = (part + 31) >> 5;
+    if (tid < part) {
+        for (int t0 = 0; t0 < slots; t0 += 4) {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            const double *p = red.partials + (size_t)t0 * kMaxReduceBlocks;
+#pragma unroll 4
+            for (int b = tid; b < (int)gridDim.x; b += part) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (t0 + q < slots) s[q] += __ldcg(p + (size_t)q * kMaxReduceBlocks + b);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (t0 + q >= slots) break;
+                s[q] = warp_sum(s[q], lane, min(active, part - warp * 32));
+                if (lane == 0) wv[warp * slots + t0 + q] = s[q];
+            }
         }
     }
     __syncthreads();
-    if (tid < n) {
-        const int r = tid;
-        double tr[NV];
+    for (int t = tid; t < slots; t += nthr) {
+        double s = 0.0;
+        for (int q = 0; q < pw; ++q) s += wv[q * slots + t];
+        slot[t] = s;
+        red.sums[t] = s;
+    }
+    __syncthreads();
+    if (red.st) {
+        for (int r = tid; r < n; r += nthr) {
+            double tr[NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            tr[k] = tots[k * n + r];
-            red.sums[k * n + r] = tr[k];
+            for (int k = 0; k < NV; ++k) tr[k] = slot[k * n + r];
+            finalize_one(red.fin, red.st + r, tr);
         }
-        if (red.st) finalize_one(red.fin, red.st + r, tr);
     }
     if (tid == 0) *red.ticket = 0u;
+}
+
+// Every one of n right-hand sides frozen.  A reducing kernel may then leave at
+// once, without its ticket: states change only in the finalize step of a last
+// block, after every block of that launch has read them here, so all blocks of
+// a launch decide alike.
+__device__ __forceinline__ bool all_frozen(const SolverState *st, int n) {
+    bool f = true;
+    for (int r = 0; r < n; ++r) f = f && st[r].stop;
+    return f;
 }
 
 // ---------------------------------------------------------------- geometry

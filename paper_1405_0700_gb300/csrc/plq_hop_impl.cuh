@@ -373,6 +373,9 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
     const long long total = (long long)a.lat.Vh * n;
     const size_t stride = (size_t)total;
     constexpr int NV = EPI == EPI_XPAY_NORM ? 1 : EPI == EPI_XPAY_DOTW ? 2 : EPI == EPI_XPAY_TS ? 3 : 0;
+    if constexpr (NV > 0) {
+        if (a.st != nullptr && all_frozen(a.st, n)) return;
+    }
     RedAcc<(NV > 0 ? NV : 1), RT> racc;
     red_init(racc);
 
@@ -428,7 +431,7 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
                 if constexpr (EPI == EPI_XPAY_NORM) {
                     T s0 = 0;
 #pragma unroll
-                    for (int k = 0; k < 12; ++k) s0 += acc[t][k].re * acc[t][k].re + acc[t][k].im * acc[t][k].im;
+                    for (int k = 0; k < 12; ++k) s0 = fma(acc[t][k].re, acc[t][k].re, fma(acc[t][k].im, acc[t][k].im, s0));
                     racc.add(0, t, s0);
                 } else if constexpr (EPI == EPI_XPAY_DOTW) {
                     cx<T> wv[12];
@@ -436,8 +439,8 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
                     T s0 = 0, s1 = 0;
 #pragma unroll
                     for (int k = 0; k < 12; ++k) {  // <w, out> = sum conj(w) out
-                        s0 += wv[k].re * acc[t][k].re + wv[k].im * acc[t][k].im;
-                        s1 += wv[k].re * acc[t][k].im - wv[k].im * acc[t][k].re;
+                        s0 = fma(wv[k].re, acc[t][k].re, fma(wv[k].im, acc[t][k].im, s0));
+                        s1 = fma(wv[k].re, acc[t][k].im, fma(-wv[k].im, acc[t][k].re, s1));
                     }
                     racc.add(0, t, s0);
                     racc.add(1, t, s1);
@@ -445,9 +448,9 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
                     T s0 = 0, s1 = 0, s2 = 0;
 #pragma unroll
                     for (int k = 0; k < 12; ++k) {  // <out, x> and |out|^2
-                        s0 += acc[t][k].re * xv[k].re + acc[t][k].im * xv[k].im;
-                        s1 += acc[t][k].re * xv[k].im - acc[t][k].im * xv[k].re;
-                        s2 += acc[t][k].re * acc[t][k].re + acc[t][k].im * acc[t][k].im;
+                        s0 = fma(acc[t][k].re, xv[k].re, fma(acc[t][k].im, xv[k].im, s0));
+                        s1 = fma(acc[t][k].re, xv[k].im, fma(-acc[t][k].im, xv[k].re, s1));
+                        s2 = fma(acc[t][k].re, acc[t][k].re, fma(acc[t][k].im, acc[t][k].im, s2));
                     }
                     racc.add(0, t, s0);
                     racc.add(1, t, s1);
@@ -565,13 +568,8 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
     const int nblk = (L.Vh + S - 1) / S;
     if (a.st != nullptr) {
         // every right-hand side frozen (a solver's iterations past convergence):
-        // nothing to stage or compute; the reduction still counts this block
-        bool all_stopped = true;
-        for (int r = 0; r < n; ++r) all_stopped = all_stopped && a.st[r].stop;
-        if (all_stopped) {
-            if constexpr (NV > 0) grid_reduce(a.red, racc, blockDim.x);
-            return;
-        }
+        // nothing to stage or compute
+        if (all_frozen(a.st, n)) return;
     }
     for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         __syncthreads();  // the previous site block is done with the shared links
@@ -748,7 +746,7 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
                 if constexpr (EPI == EPI_XPAY_NORM) {
                     T s0 = 0;
 #pragma unroll
-                    for (int e = 0; e < 12; ++e) s0 += acc[t][e].re * acc[t][e].re + acc[t][e].im * acc[t][e].im;
+                    for (int e = 0; e < 12; ++e) s0 = fma(acc[t][e].re, acc[t][e].re, fma(acc[t][e].im, acc[t][e].im, s0));
                     racc.add(0, t, s0);
                 }
             }
