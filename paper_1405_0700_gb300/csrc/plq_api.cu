@@ -35,7 +35,14 @@ plq_status launch_hop_f16_12(const HopArgs &a, int epi, cudaStream_t s, int bloc
 
 int hop_default_block(int prec) { return prec == PLQ_F64 ? 128 : 128; }
 
-plq_status launch_hop(const HopArgs &a, int prec, int reals, int epi, cudaStream_t s) {
+plq_status launch_hop(const HopArgs &args, int prec, int reals, int epi, cudaStream_t s) {
+    HopArgs a = args;
+    a.a32 = (float)a.a;
+    a.nu_x32 = (float)a.nu_x;
+    a.nu_h32 = (float)a.nu_h;
+    a.scale_h32 = (float)a.scale_h;
+    a.twist_x = a.nu_x != 0.0;
+    a.twist_h = a.nu_h != 0.0 || a.scale_h != 1.0;
     const int block = a.block > 0 ? a.block : hop_default_block(prec);
     const bool r12 = reals == 12;
     switch (prec) {

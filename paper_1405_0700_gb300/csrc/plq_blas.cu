@@ -38,6 +38,18 @@ __device__ __forceinline__ int rhs_of(long long e, int n) { return n == 1 ? 0 : 
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)(N); \
          e += (long long)gridDim.x * blockDim.x)
 
+// A solver coefficient in the arithmetic of the kernel.
+template <class T>
+__device__ __forceinline__ T coef(double d, float f) {
+    if constexpr (sizeof(T) == 4) return f;
+    else return d;
+}
+template <class T>
+__device__ __forceinline__ cx<T> coef(double2 d, float2 f) {
+    if constexpr (sizeof(T) == 4) return {f.x, f.y};
+    else return {d.x, d.y};
+}
+
 template <class A, class B>
 __device__ __forceinline__ void convert(const cx<A> in[12], cx<B> out[12]) {
 #pragma unroll
@@ -129,7 +141,7 @@ __global__ void cg_update_kernel(long long N, int n, void *x, void *r, const voi
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
         if (st[rr].stop) continue;
-        const T alpha = (T)st[rr].alpha;
+        const T alpha = coef<T>(st[rr].alpha, st[rr].alpha32);
         cx<T> pv[12], qv[12], rv[12];
         cx<TX> xv[12];
         Spinor<P>::load(p, N, e, pv);
@@ -159,7 +171,7 @@ __global__ void cg_direction_kernel(long long N, int n, void *p, const void *r, 
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
         if (st[rr].stop) continue;
-        const T beta = (T)st[rr].beta;
+        const T beta = coef<T>(st[rr].beta, st[rr].beta32);
         cx<T> pv[12], rv[12];
         Spinor<P>::load(p, N, e, pv);
         Spinor<P>::load(r, N, e, rv);
@@ -266,9 +278,8 @@ __global__ void xpay64_kernel(long long N, const void *x, double a, void *y) {
 }
 
 template <class T>
-__device__ __forceinline__ cx<T> cmulc(double2 c, cx<T> z) {
-    const T a = (T)c.x, b = (T)c.y;
-    return {a * z.re - b * z.im, a * z.im + b * z.re};
+__device__ __forceinline__ cx<T> cmulc(cx<T> c, cx<T> z) {
+    return {c.re * z.re - c.im * z.im, c.re * z.im + c.im * z.re};
 }
 
 // p = r + beta (p - omega v)
@@ -278,7 +289,7 @@ __global__ void bicg_p_kernel(long long N, int n, void *p, const void *r, const 
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
         if (st[rr].stop) continue;
-        const double2 beta = st[rr].c_beta, omega = st[rr].c_omega;
+        const cx<T> beta = coef<T>(st[rr].c_beta, st[rr].c_beta32), omega = coef<T>(st[rr].c_omega, st[rr].c_omega32);
         cx<T> pv[12], rv[12], vv[12];
         Spinor<P>::load(p, N, e, pv);
         Spinor<P>::load(r, N, e, rv);
@@ -296,7 +307,7 @@ __global__ void bicg_s_kernel(long long N, int n, void *s, const void *r, const 
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
         if (st[rr].stop) continue;
-        const double2 alpha = st[rr].c_alpha;
+        const cx<T> alpha = coef<T>(st[rr].c_alpha, st[rr].c_alpha32);
         cx<T> rv[12], vv[12];
         Spinor<P>::load(r, N, e, rv);
         Spinor<P>::load(v, N, e, vv);
@@ -318,7 +329,7 @@ __global__ void bicg_update_kernel(long long N, int n, void *x, void *r, const v
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
         if (st[rr].stop) continue;
-        const double2 alpha = st[rr].c_alpha, omega = st[rr].c_omega;
+        const cx<T> alpha = coef<T>(st[rr].c_alpha, st[rr].c_alpha32), omega = coef<T>(st[rr].c_omega, st[rr].c_omega32);
         cx<T> pv[12], sv[12], tv[12], hv[12];
         cx<TX> xv[12];
         Spinor<P>::load(p, N, e, pv);

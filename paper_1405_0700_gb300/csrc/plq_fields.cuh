@@ -299,8 +299,11 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
 // Finalize step of one right-hand side's reduction: update its solver
-// scalars in device memory from the grid totals tot[0..NV).
-__device__ __forceinline__ void finalize_one(int fin, SolverState *st, const double *tot) {
+// scalars from the grid totals tot[0..NV).  The state is read, changed and
+// written back as a whole: its fields are then one L2 round trip, not one for
+// every field that a store to another might alias.
+__device__ __forceinline__ void finalize_one(int fin, SolverState *state, const double *tot) {
+    SolverState z = *state, *st = &z;
     // A frozen right-hand side contributed nothing to this reduction: its
     // scalars must not change.
     if (st->stop) return;
@@ -308,12 +311,14 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *st, const dou
     case FIN_CG_ALPHA:
         st->pAp = tot[0];
         st->alpha = st->rho / tot[0];
+        st->alpha32 = (float)st->alpha;
         if (!isfinite(st->alpha)) { st->flags |= FLAG_NAN; st->stop = 1; }
         if (st->hist && st->iter < st->hist_cap) st->hist[3 * st->iter] = st->alpha;
         break;
     case FIN_CG_BETA:
         st->rho_new = tot[0];
         st->beta = tot[0] / st->rho;
+        st->beta32 = (float)st->beta;
         st->rho = tot[0];
         if (st->hist && st->iter < st->hist_cap) {
             st->hist[3 * st->iter + 1] = st->beta;
@@ -328,6 +333,7 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *st, const dou
         const double m = fabs(tot[0]) + fabs(tot[1]);
         if (!(m > st->tiny)) { st->flags |= (isfinite(m) ? FLAG_BREAKDOWN : FLAG_NAN); st->stop = 1; break; }
         st->c_alpha = cdiv(st->c_rho, st->rv);
+        st->c_alpha32 = make_float2((float)st->c_alpha.x, (float)st->c_alpha.y);
         break;
     }
     case FIN_BICG_OMEGA:
@@ -339,6 +345,7 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *st, const dou
             break;
         }
         st->c_omega = make_double2(tot[0] / tot[2], tot[1] / tot[2]);
+        st->c_omega32 = make_float2((float)st->c_omega.x, (float)st->c_omega.y);
         if (fabs(st->c_omega.x) + fabs(st->c_omega.y) == 0.0) { st->flags |= FLAG_BREAKDOWN; st->stop = 1; }
         break;
     case FIN_BICG_RHO: {
@@ -349,6 +356,7 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *st, const dou
         if (tot[2] <= st->stop_r2 || st->iter >= st->maxit) { st->stop = 1; st->c_rho_new = rn; break; }
         if (!(fabs(rn.x) + fabs(rn.y) > 0.0)) { st->flags |= FLAG_BREAKDOWN; st->stop = 1; break; }
         st->c_beta = cmul(cdiv(rn, st->c_rho), cdiv(st->c_alpha, st->c_omega));
+        st->c_beta32 = make_float2((float)st->c_beta.x, (float)st->c_beta.y);
         st->c_rho = rn;
         st->c_rho_new = rn;
         break;
@@ -356,6 +364,7 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *st, const dou
     default:
         break;
     }
+    *state = z;
 }
 
 // Per-thread FP64 accumulator of NV sums for the RT right-hand sides a thread
@@ -398,73 +407,118 @@ __device__ __forceinline__ V warp_sum(V x, int lane, int active) {
     return x;
 }
 
-// Combine the accumulators of the whole grid (ncols right-hand-side columns
-// of RT right-hand sides each): within a warp the lanes of each column are
-// folded onto its first lanes; the warps' column sums are added in warp order,
-// kRedWarps warps per block barrier; each block writes its partial sums to
-// red.partials, and the last block to finish (ticket counter) adds them, every
-// thread striding over the blocks, stores the totals in red.sums[k*n + r] and
-// applies the finalize step to red.st[r].  The order is fixed for a launch
-// configuration.  Every thread of every block must call it.
+// Block sums of the RedAcc values: total (value v, column c) goes to
+// slot[(k*n + c*RT) + t], v = k*RT + t, valid for every thread after the
+// closing barrier.  wv: kRedThreads * W doubles (W <= 4) or 32 * (warps) (W = 32).
 //
-// This tail is latency, not bandwidth: what counts is the chain of barriers,
-// fences and L2 round trips behind the last site.  So one thread fences for
-// its block (the barrier before it orders the other threads' stores), the
-// partial sums of a slot lie side by side (the last block reads 256 blocks in
-// one coalesced load per slot), and all loads of a slot group are in flight
-// together.  Measured as launches with no element to work on (all right-hand
-// sides frozen, 24^3x48): see grid_reduce figures at all_frozen().
-constexpr int kRedWarps = 8;
+// An FP64 warp instruction occupies this GPU's FP64 pipe for 15 cycles (2.1
+// results per clock and SM), so what a reduction costs is its number of FP64
+// warp instructions.  A shuffle tree in each of 8 warps takes 40 per value;
+// here the threads store their values and one warp per value adds 8 of them
+// per lane before a single tree: 13.  Wide sums (W = 32 values, one column)
+// use recursive halving in each warp, 31 additions instead of 160.
+constexpr int kRedThreads = 256;
 
 template <int NV, int RT>
+__device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols, double *wv, double *slot) {
+    constexpr int W = NV * RT;
+    const int tid = ltid(), lane = tid & 31, warp = tid >> 5, nthr = lsize(), nw = (nthr + 31) >> 5;
+    const int n = ncols * RT;
+    if constexpr (W == 32) {  // one column, whole warps
+        double x[W];
+#pragma unroll
+        for (int k = 0; k < W; ++k) x[k] = w[k];
+#pragma unroll
+        for (int h = 16; h >= 1; h >>= 1) {
+            const bool up = (lane & h) != 0;
+#pragma unroll
+            for (int k = 0; k < h; ++k) {
+                // lanes without bit h keep value k, the others value k + h
+                const double give = up ? x[k] : x[k + h];
+                const double keep = up ? x[k + h] : x[k];
+                x[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+            }
+        }
+        wv[warp * 32 + lane] = x[0];  // lane l holds value l
+        __syncthreads();
+        if (tid < 32) {
+            double s = 0.0;
+            for (int q = 0; q < nw; ++q) s += wv[q * 32 + tid];
+            slot[tid] = s;
+        }
+        __syncthreads();
+    } else {
+        // warps that add: the full ones, or the only one
+        const int full = nthr >= 32 ? nthr >> 5 : 1, lanes = min(32, nthr);
+        const int per = lanes / ncols;  // lanes per column
+        const int c = lane % ncols, part = lane / ncols;
+        for (int v0 = 0; v0 < W; v0 += full) {  // (a block of fewer warps than values goes round again)
+            const int v = v0 + warp;
+            const bool adds = warp < full && v < W;
+            double s = 0.0;
+            for (int base = 0; base < nthr; base += kRedThreads) {
+                if (v0 > 0 || base > 0) __syncthreads();
+                if (tid >= base && tid < base + kRedThreads) {
+#pragma unroll
+                    for (int k = 0; k < W; ++k) wv[k * kRedThreads + tid - base] = w[k];
+                }
+                __syncthreads();
+                if (adds && part < per) {
+                    int i = (c - base) % ncols;  // first thread of the round in column c
+                    if (i < 0) i += ncols;
+                    const int cnt = min(kRedThreads, nthr - base);
+                    for (i += part * ncols; i < cnt; i += per * ncols) s += wv[v * kRedThreads + i];
+                }
+            }
+            if (adds) {
+                const unsigned mask = lanes >= 32 ? 0xffffffffu : ((1u << lanes) - 1u);
+                int o = 1;
+                while (2 * o < per) o *= 2;
+                if (per > 1)
+                    for (; o >= 1; o >>= 1) {
+                        const double y = __shfl_down_sync(mask, s, o * ncols);
+                        if (part < o && part + o < per) s += y;
+                    }
+                if (part == 0) {
+                    const int k = v / RT;
+                    slot[k * n + c * RT + (v - k * RT)] = s;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Combine the accumulators of the whole grid (ncols right-hand-side columns
+// of RT right-hand sides each): each block writes its sums to red.partials,
+// and the last block to finish (ticket counter) adds them, stores the totals
+// in red.sums[k*n + r] and applies the finalize step to red.st[r].  The order
+// is fixed for a launch configuration.  Every thread of every block must call it.
+//
+// Behind the last site this is a chain of barriers, fences and L2 round trips:
+// one thread fences for its block (the barrier before it orders the other
+// threads' stores), the partial sums of a slot lie side by side (the last
+// block reads 256 blocks in one coalesced load per slot), and the loads of a
+// slot group are in flight together.  Measured (with the early exit of
+// all_frozen and the FP32 coefficients of SolverState): mixed BiCGstab on
+// 20x12x28x36 8.10 -> 5.46 ms, EigCG on 16^3x32 303 -> 272 ms (its 32-value
+// sums 234 -> 130 us), FP64 norm of a 24^3x48 half field 35 -> 25 us.
+template <int NV, int RT>
 __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int ncols) {
-    constexpr int W = NV * RT;                      // values per thread
-    constexpr int kCols = W > 4 ? 1 : PLQ_MAX_RHS;  // columns that fit wv (the wide forms have one)
-    __shared__ double wv[kRedWarps * kCols * W];    // (warp of the round, lane, value), later (warp, slot)
+    constexpr int W = NV * RT;
+    constexpr int kWords = W == 32 ? 32 * 32 : W * kRedThreads;
+    __shared__ double wv[kWords];
     __shared__ double slot[kPartialSlots];
     __shared__ bool last;
-    const int tid = ltid(), lane = tid & 31, warp = tid >> 5, nthr = lsize(), nw = (nthr + 31) >> 5;
-    const int active = min(32, nthr - warp * 32);  // lanes present in this thread's warp
+    const int tid = ltid(), nthr = lsize();
     const int n = ncols * RT, slots = NV * n;
     double w[W];
 #pragma unroll
     for (int k = 0; k < NV; ++k)
 #pragma unroll
         for (int t = 0; t < RT; ++t) w[k * RT + t] = acc.v[k][t];
-    if (ncols == 1) {
-#pragma unroll
-        for (int k = 0; k < W; ++k) w[k] = warp_sum(w[k], lane, active);
-    } else {
-        const unsigned mask = active >= 32 ? 0xffffffffu : ((1u << active) - 1u);
-        for (int o = ncols; o < 32; o += ncols) {
-#pragma unroll
-            for (int k = 0; k < W; ++k) {
-                const double y = __shfl_down_sync(mask, w[k], o);
-                if (lane < ncols && lane + o < active) w[k] += y;
-            }
-        }
-    }
-    for (int t = tid; t < slots; t += nthr) slot[t] = 0.0;
-    for (int w0 = 0; w0 < nw; w0 += kRedWarps) {
-        if (w0 > 0) __syncthreads();
-        if (warp >= w0 && warp < w0 + kRedWarps && lane < min(ncols, active)) {
-#pragma unroll
-            for (int k = 0; k < W; ++k) wv[((warp - w0) * ncols + lane) * W + k] = w[k];
-        }
-        __syncthreads();
-        const int w1 = min(nw, w0 + kRedWarps);
-        for (int t = tid; t < slots; t += nthr) {  // (a slot stays with its thread)
-            const int k = t / n, c = (t - k * n) / RT, v = k * RT + (t - k * n) - c * RT;
-            double s = slot[t];
-            for (int ww = w0; ww < w1; ++ww) {
-                int l = c - (32 * ww) % ncols;  // the lane of warp ww that holds column c
-                if (l < 0) l += ncols;
-                if (l < nthr - 32 * ww) s += wv[((ww - w0) * ncols + l) * W + v];
-            }
-            slot[t] = s;
-            if (w1 == nw) red.partials[(size_t)t * kMaxReduceBlocks + blockIdx.x] = s;
-        }
-    }
+    block_sums<NV, RT>(w, ncols, wv, slot);
+    for (int t = tid; t < slots; t += nthr) red.partials[(size_t)t * kMaxReduceBlocks + blockIdx.x] = slot[t];
     __syncthreads();
     if (tid == 0) {
         __threadfence();
@@ -473,15 +527,21 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int nc
     }
     __syncthreads();
     if (!last) return;
-    // The last block: its first kRedWarps warps stride over the blocks, four
-    // slots at a time, then the warps' sums are added in warp order.
-    const int part = min(nthr, 32 * kRedWarps), pw = (part + 31) >> 5;
-    if (tid < part) {
-        for (int t0 = 0; t0 < slots; t0 += 4) {
+    if (ncols == 1) {
+#pragma unroll
+        for (int q = 0; q < W; ++q) w[q] = 0.0;
+#pragma unroll 4
+        for (int b = tid; b < (int)gridDim.x; b += nthr) {
+#pragma unroll
+            for (int q = 0; q < W; ++q) w[q] += __ldcg(red.partials + (size_t)q * kMaxReduceBlocks + b);
+        }
+        block_sums<W, 1>(w, 1, wv, slot);
+    } else if constexpr (W <= 4) {
+        for (int t0 = 0; t0 < slots; t0 += 4) {  // the loads of four slots in flight together
             double s[4] = {0.0, 0.0, 0.0, 0.0};
             const double *p = red.partials + (size_t)t0 * kMaxReduceBlocks;
 #pragma unroll 4
-            for (int b = tid; b < (int)gridDim.x; b += part) {
+            for (int b = tid; b < (int)gridDim.x; b += nthr) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (t0 + q < slots) s[q] += __ldcg(p + (size_t)q * kMaxReduceBlocks + b);
@@ -489,19 +549,12 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int nc
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (t0 + q >= slots) break;
-                s[q] = warp_sum(s[q], lane, min(active, part - warp * 32));
-                if (lane == 0) wv[warp * slots + t0 + q] = s[q];
+                const double one[1] = {s[q]};
+                block_sums<1, 1>(one, 1, wv, slot + t0 + q);
             }
         }
     }
-    __syncthreads();
-    for (int t = tid; t < slots; t += nthr) {
-        double s = 0.0;
-        for (int q = 0; q < pw; ++q) s += wv[q * slots + t];
-        slot[t] = s;
-        red.sums[t] = s;
-    }
-    __syncthreads();
+    for (int t = tid; t < slots; t += nthr) red.sums[t] = slot[t];
     if (red.st) {
         for (int r = tid; r < n; r += nthr) {
             double tr[NV];

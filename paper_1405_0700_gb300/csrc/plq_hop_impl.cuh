@@ -37,6 +37,28 @@ __device__ __forceinline__ void twist12(cx<T> v[12], T nu, T scale) {
     }
 }
 
+// Scalars of a launch in the arithmetic of the kernel.
+template <class T>
+__device__ __forceinline__ T hop_a(const HopArgs &a) {
+    if constexpr (sizeof(T) == 4) return a.a32;
+    else return a.a;
+}
+template <class T>
+__device__ __forceinline__ T hop_nu_x(const HopArgs &a) {
+    if constexpr (sizeof(T) == 4) return a.nu_x32;
+    else return a.nu_x;
+}
+template <class T>
+__device__ __forceinline__ T hop_nu_h(const HopArgs &a) {
+    if constexpr (sizeof(T) == 4) return a.nu_h32;
+    else return a.nu_h;
+}
+template <class T>
+__device__ __forceinline__ T hop_scale_h(const HopArgs &a) {
+    if constexpr (sizeof(T) == 4) return a.scale_h32;
+    else return a.scale_h;
+}
+
 template <int MU>
 struct Proj;
 template <>
@@ -417,12 +439,12 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
             const int rr = r0 + t;
             if (RT > 1 && a.st != nullptr && a.st[rr].stop) continue;
             const long long idx = PLQ_GUARD(a.kstatus, (long long)i * n + rr, (long long)stride);
-            if (a.nu_h != 0.0 || a.scale_h != 1.0) twist12(acc[t], (T)a.nu_h, (T)a.scale_h);
+            if (a.twist_h) twist12(acc[t], hop_nu_h<T>(a), hop_scale_h<T>(a));
             if constexpr (EPI != EPI_PLAIN) {
                 cx<T> xv[12];
                 Spinor<P>::load(a.x, stride, (size_t)idx, xv);
-                if (a.nu_x != 0.0) twist12(xv, (T)a.nu_x, T(1));
-                const T s = (T)a.a;
+                if (a.twist_x) twist12(xv, hop_nu_x<T>(a), T(1));
+                const T s = hop_a<T>(a);
 #pragma unroll
                 for (int k = 0; k < 12; ++k) {
                     acc[t][k].re = fma(s, acc[t][k].re, xv[k].re);
@@ -732,12 +754,12 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
             const int rr = r0 + t;
             if (a.st != nullptr && a.st[rr].stop) continue;
             const long long idx = PLQ_GUARD(a.kstatus, (long long)i * n + rr, (long long)stride);
-            if (a.nu_h != 0.0 || a.scale_h != 1.0) twist12(acc[t], (T)a.nu_h, (T)a.scale_h);
+            if (a.twist_h) twist12(acc[t], hop_nu_h<T>(a), hop_scale_h<T>(a));
             if constexpr (EPI != EPI_PLAIN) {
                 cx<T> xv[12];
                 Spinor<P>::load(a.x, stride, (size_t)idx, xv);
-                if (a.nu_x != 0.0) twist12(xv, (T)a.nu_x, T(1));
-                const T s = (T)a.a;
+                if (a.twist_x) twist12(xv, hop_nu_x<T>(a), T(1));
+                const T s = hop_a<T>(a);
 #pragma unroll
                 for (int e = 0; e < 12; ++e) {
                     acc[t][e].re = fma(s, acc[t][e].re, xv[e].re);

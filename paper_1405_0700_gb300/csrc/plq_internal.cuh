@@ -111,6 +111,11 @@ struct SolverState {
     double *hist;
     int hist_cap;
     int pad2;
+    // The coefficients as FP32 kernels use them, converted once where they are
+    // computed: a conversion costs every warp that makes it 15 cycles of the
+    // FP64 pipe.
+    float alpha32, beta32;
+    float2 c_alpha32, c_omega32, c_beta32;
 };
 
 enum { FLAG_NAN = 1, FLAG_BREAKDOWN = 2 };
@@ -251,6 +256,11 @@ struct HopArgs {
     // replaced by scale_h * (1 + i nu_h gamma5) H in, and the xpay source x by
     // (1 + i nu_x gamma5) x.
     double nu_x = 0.0, nu_h = 0.0, scale_h = 1.0;
+    // The same scalars as FP32-arithmetic kernels use them, and which twists
+    // are present (set by launch_hop): FP64 conversions and comparisons in the
+    // kernel would take 15 cycles of the FP64 pipe per warp and site.
+    float a32 = 0.f, nu_x32 = 0.f, nu_h32 = 0.f, scale_h32 = 1.f;
+    int twist_x = 0, twist_h = 0;
     int site_begin = 0;   // output sites [site_begin, site_end) of the parity;
     int site_end = -1;    // -1: up to Vh
     int smem_links = 0;   // multi-RHS: stage each block's links in shared memory

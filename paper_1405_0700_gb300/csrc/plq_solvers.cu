@@ -354,6 +354,7 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     // p = r_true + beta p, beta = |r_true|^2 / rho_k with rho_k the
                     // |r|^2 of the iteration before the one that triggered.
                     init[r].beta = first ? 0.0 : r2[r] / last_rho[r];
+                    init[r].beta32 = (float)init[r].beta;
                     init[r].stop_r2 = std::fmax(delta * delta * r2[r], target2[r]);
                 }
                 if ((st = put_states(S, init)) != PLQ_OK) break;
