@@ -8,7 +8,8 @@ from oracle import c_oracle as C
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_1405_0700_gb300 import F32, F64, Context  # noqa: E402
+from paper_1405_0700_gb300 import F16, F32, F64, Context, PLQError  # noqa: E402
+from paper_1405_0700_gb300 import plq  # noqa: E402
 
 
 # grids of one block and of many, blocks of one warp, of a partial last warp and of more
@@ -38,3 +39,59 @@ def test_grid_reductions(dims, nrhs, block, tile, method):
         # both residuals are FP64 sums over the same x: they differ by the rounding of M x,
         # of order 1e-16 of |b|
         assert abs(infos[r].true_rel_residual - res) < 1e-13
+
+
+# blocks that hold fewer pairs of sites than the lattice leaves them (4x2x2x2: one block;
+# 6x10x2x14: ragged last blocks), one to twelve right-hand sides
+@pytest.mark.parametrize("dims", [(4, 2, 2, 2), (6, 10, 2, 14), (4, 6, 4, 2)])
+@pytest.mark.parametrize("nrhs", [1, 2, 5, 12])
+@pytest.mark.parametrize("prec", [F64, F32, F16])
+def test_pack_and_unpack(dims, nrhs, prec):
+    T, Lx, Ly, Lz = dims
+    rng = np.random.default_rng(7)
+    phi = rng.standard_normal((nrhs, T, Lz, Ly, Lx, 12, 2)).view(np.complex128)[..., 0]
+    t, z, y, x = np.meshgrid(*[np.arange(k) for k in (T, Lz, Ly, Lx)], indexing="ij")
+    parity = (t + x + y + z) % 2
+    with Context(dims) as ctx:
+        full = ctx.to_device(phi if nrhs > 1 else phi[0], prec, nrhs)
+        back = ctx.to_host(full, prec, nrhs).reshape(phi.shape[:5] + (12,))
+        halves = [h.cpu().numpy() for h in ctx.halves(full, prec, nrhs)]
+    Vh = T * Lx * Ly * Lz // 2
+    for p in (0, 1):
+        ref = phi[:, parity == p].transpose(1, 0, 2)  # (Vh, nrhs, 12): sites in checkerboard order
+        if prec == F64:
+            got = halves[p].view(np.float64).reshape(12, Vh, nrhs, 2)
+            assert np.array_equal(got[..., 0] + 1j * got[..., 1], ref.transpose(2, 0, 1))
+        elif prec == F32:
+            got = halves[p].view(np.float32).reshape(6, Vh, nrhs, 2, 2).transpose(1, 2, 0, 3, 4).reshape(Vh, nrhs, 12, 2)
+            assert np.array_equal(got, ref.astype(np.complex64).view(np.float32).reshape(Vh, nrhs, 12, 2))
+        else:
+            norms = halves[p][48 * Vh * nrhs:].view(np.float32).reshape(Vh, nrhs)
+            r32 = ref.astype(np.complex64).view(np.float32).reshape(Vh, nrhs, 24)
+            assert np.array_equal(norms, np.abs(r32).max(axis=2))
+    # FP64 exact; FP32 to half an ulp; FP16 to half an ulp of the site's largest component
+    tol = {F64: 0.0, F32: 2.0**-24, F16: 2.0**-10}[prec]
+    assert np.abs(back - phi).max() <= tol * np.sqrt(2) * np.abs(phi).max()
+
+
+@pytest.mark.parametrize("what,accepted", [("none", True), ("1e-11 in row 0", False), ("1e-11 in row 2", False),
+                                           ("5e-13 in row 2", True), ("1e-11 row 1 phase", False)])
+@pytest.mark.parametrize("dims", [(4, 2, 2, 2), (2, 6, 4, 10)])
+def test_su3_check_of_twelve_real_links(what, accepted, dims):
+    U = S.gauge_field(dims, 0.3, 3)
+    u = U[-1, -1, -1, -1, 3]  # the last link of the lattice
+    if what == "1e-11 in row 0":
+        u[0, 1] += 1e-11
+    elif what == "1e-11 in row 2":
+        u[2, 2] += 1e-11j
+    elif what == "5e-13 in row 2":  # below the limit, above the short test's
+        u[2, 0] += 5e-13 * u[2, 1] / abs(u[2, 1])
+    elif what == "1e-11 row 1 phase":  # rows stay orthonormal, row 2 no longer their product
+        u[1] *= np.exp(1e-11j)
+    with Context(dims) as ctx:
+        if accepted:
+            ctx.gauge_upload(U, 12, F32)
+        else:
+            with pytest.raises(PLQError) as e:
+                ctx.gauge_upload(U, 12, F32)
+            assert e.value.status == plq.PLQ_ERR_ARG
