@@ -480,7 +480,11 @@ typedef struct {
                              neighbour spinors copied into a ring of shared-memory slots
                              by bulk (TMA) copies, sites_per_thread then being the number
                              of slots (0: as many as fit); set by plq_set_launch only
-                             (the tuner does not time it: slower on GB300)             */
+                             (the tuner does not time it: slower on GB300);
+                             5 split kernel, the eight directions of a site on eight
+                             warps: the library's own choice for FP64 storage and small
+                             lattices, and a candidate of the tuner (plq_set_launch
+                             does not take it: all zeros leave the choice to the library) */
     double us_per_launch; /* measured time of one half-lattice application                 */
     int from_cache;       /* 1 if the choice came from the cache file                      */
     int candidates;       /* configurations timed                                          */

@@ -163,9 +163,8 @@ struct Spinor<PLQ_F16> {
         }
         return ld_nc(nrm + e);
     }
-    __device__ static void store(void *base, size_t stride, size_t e, const cx<float> v[12]) {
-        uint4 *p = static_cast<uint4 *>(base) + e;
-        float *nrm = reinterpret_cast<float *>(static_cast<uint4 *>(base) + 3 * stride);
+    // Site norm of v, and its inverse (0 for a site stored as zero).
+    __device__ static float site_norm(const cx<float> v[12], float &inv) {
         float m = 0.f;
 #pragma unroll
         for (int k = 0; k < 12; ++k) m = fmaxf(m, fmaxf(fabsf(v[k].re), fabsf(v[k].im)));
@@ -175,17 +174,33 @@ struct Spinor<PLQ_F16> {
         // of a point source, many orders of magnitude below the field's norm.
         constexpr float kMinNormal = 1.17549435e-38f;
         if (!(m >= kMinNormal)) m = 0.f;
-        const float inv = m > 0.f ? 1.0f / m : 0.f;
+        inv = m > 0.f ? 1.0f / m : 0.f;
+        return m;
+    }
+    __device__ static uint4 halves(const cx<float> v[4], float inv) {
+        uint4 t;
+        t.x = f2h(v[0].re * inv, v[0].im * inv);
+        t.y = f2h(v[1].re * inv, v[1].im * inv);
+        t.z = f2h(v[2].re * inv, v[2].im * inv);
+        t.w = f2h(v[3].re * inv, v[3].im * inv);
+        return t;
+    }
+    __device__ static void store(void *base, size_t stride, size_t e, const cx<float> v[12]) {
+        uint4 *p = static_cast<uint4 *>(base) + e;
+        float inv;
+        const float m = site_norm(v, inv);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            uint4 t;
-            t.x = f2h(v[4 * k + 0].re * inv, v[4 * k + 0].im * inv);
-            t.y = f2h(v[4 * k + 1].re * inv, v[4 * k + 1].im * inv);
-            t.z = f2h(v[4 * k + 2].re * inv, v[4 * k + 2].im * inv);
-            t.w = f2h(v[4 * k + 3].re * inv, v[4 * k + 3].im * inv);
-            __stcs(p + k * stride, t);
-        }
-        __stcs(nrm + e, m);
+        for (int k = 0; k < 3; ++k) __stcs(p + k * stride, halves(v + 4 * k, inv));
+        __stcs(reinterpret_cast<float *>(static_cast<uint4 *>(base) + 3 * stride) + e, m);
+    }
+    // One of the three planes (plane 0 with the norm).
+    __device__ static void store_plane(void *base, size_t stride, size_t e, const cx<float> v[12], int k) {
+        float inv;
+        const float m = site_norm(v, inv);
+        const cx<float> q[4] = {k == 0 ? v[0] : k == 1 ? v[4] : v[8], k == 0 ? v[1] : k == 1 ? v[5] : v[9],
+                                k == 0 ? v[2] : k == 1 ? v[6] : v[10], k == 0 ? v[3] : k == 1 ? v[7] : v[11]};
+        static_cast<uint4 *>(base)[k * stride + e] = halves(q, inv);
+        if (k == 0) reinterpret_cast<float *>(static_cast<uint4 *>(base) + 3 * stride)[e] = m;
     }
 };
 

@@ -910,6 +910,7 @@ plq_status dispatch_tiled(const HopArgs &a, int epi, cudaStream_t s, int block) 
 }  // namespace plq
 
 #include "plq_hop_rows.cuh"
+#include "plq_hop_split.cuh"
 
 namespace plq {
 
@@ -919,6 +920,14 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
     // formats and the epilogues of operator applications and CG; the
     // neighbour-table variants for the plain and xpay epilogues; the
     // row-streamed kernel for whole-lattice applications with those epilogues.
+    if (a.smem_links == 5 || a.untuned) {
+        if (split_fits(a, epi) && (a.smem_links == 5 || split_default<P>(a))) return dispatch_split<P, R>(a, epi, s);
+        if (a.smem_links == 5) {  // a tuned split launch, where the split kernel has no form: the library's default
+            HopArgs d = a;
+            d.smem_links = d.block = 0;
+            return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
+        }
+    }
     if constexpr (P != PLQ_F64) {
         if (a.smem_links == 4 && a.site_begin == 0 && a.site_end < 0 && epi <= EPI_XPAY_NORM)
             return dispatch_rows<P, R>(a, epi, s);

@@ -268,6 +268,7 @@ struct HopArgs {
     // thread walks its share of the sites); k > 0 = enough blocks for k sites
     // (site blocks of the multi-RHS kernel) per thread.
     int spt = 0;
+    int untuned = 0;  // the launch entry of (prec, nrhs) holds no choice: the library picks kernel and shape
     // Bounded waits of the row-streamed kernel: a wait gives up after
     // spin_limit clock cycles and records PLQ_ERR_TIMEOUT in *kstatus.
     long long spin_limit = 1LL << 40;

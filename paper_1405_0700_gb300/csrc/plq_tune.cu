@@ -54,7 +54,7 @@ bool cache_lookup(const char *path, const std::string &key, TuneEntry *e) {
         // key block index_mode rhs_tile z_chunk smem_links us [sites_per_thread]
         const int got = sscanf(line, "%599s %d %d %d %d %d %f %d", k, &block, &mode, &tile, &zc, &sm, &us, &spt);
         const bool valid = (block == 0 || (block >= 32 && block <= 1024 && block % 32 == 0)) && (mode == 0 || mode == 1) &&
-                           (tile == 1 || tile == 2 || tile == 4) && zc >= 0 && sm >= 0 && sm <= 4 && spt >= 0 &&
+                           (tile == 1 || tile == 2 || tile == 4) && zc >= 0 && sm >= 0 && sm <= 5 && spt >= 0 &&
                            spt <= 64 && !(sm >= 2 && tile != 1) && !(sm == 1 && tile == 4);
         if (got >= 7 && key == k && valid) {
             e->block = block;
@@ -100,8 +100,9 @@ void apply_tune(const Ctx *c, int prec, int nrhs, HopArgs &a) {
     a.nbr = (e.index_mode == 1) ? c->nbr[a.out_parity] : nullptr;
     a.rhs_tile = (e.rhs_tile > 1 && nrhs % e.rhs_tile == 0) ? e.rhs_tile : 1;
     a.zc = (e.zc > 0 && c->lat.L[3] % e.zc == 0) ? e.zc : 0;
-    a.smem_links = (nrhs > 1 || e.smem_links == 4) ? e.smem_links : 0;
+    a.smem_links = (nrhs > 1 || e.smem_links >= 4) ? e.smem_links : 0;
     a.spt = e.spt;
+    a.untuned = e.block == 0 && e.index_mode == 0 && e.rhs_tile <= 1 && e.zc == 0 && e.smem_links == 0 && e.spt == 0;
     a.kstatus = c->kstatus;
     if (c->spin_limit > 0) a.spin_limit = c->spin_limit;
 }
@@ -233,10 +234,22 @@ extern "C" plq_status plq_autotune(plq_ctx *c, int prec, int nrhs, const char *c
             }
         }
     }
+    // the split kernel (its block and grid are its own)
+    if (st == PLQ_OK) {
+        TuneEntry t;
+        t.block = 256;
+        t.smem_links = 5;
+        float us = -1.f;
+        st = time_cfg(t, &us);
+        if (st == PLQ_OK && us >= 0.f && us < best.us) {
+            t.us = us;
+            best = t;
+        }
+    }
     // sites per thread: a grid sized for k sites (site blocks) per thread
     // against the one-wave grid of the sweep above
     for (int k : {1, 2, 4, 8}) {
-        if (st != PLQ_OK) break;
+        if (st != PLQ_OK || best.smem_links == 5) break;
         TuneEntry t = best;
         t.spt = k;
         float us = -1.f;

@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 
 import synthetic as S
+from gpuhelp import TOL, gpu_hopping_full, rel
 from oracle import c_oracle as C
 
 torch = pytest.importorskip("torch")
@@ -95,3 +96,35 @@ def test_su3_check_of_twelve_real_links(what, accepted, dims):
             with pytest.raises(PLQError) as e:
                 ctx.gauge_upload(U, 12, F32)
             assert e.value.status == plq.PLQ_ERR_ARG
+
+
+# the split kernel (eight warps per 32 elements), the default for FP64 storage and small
+# lattices: a last block of fewer elements (16 sites; 5 right-hand sides), the largest FP32
+# lattice it takes and the first it does not, and an odd number of sites per block
+@pytest.mark.parametrize("dims,nrhs", [((4, 2, 2, 2), 1), ((2, 2, 2, 4), 5), ((6, 10, 2, 6), 1), ((16, 8, 8, 16), 1),
+                                       ((16, 10, 8, 14), 1), ((4, 4, 6, 4), 12)])
+@pytest.mark.parametrize("prec,reals", [(F64, 18), (F64, 12), (F32, 18), (F32, 12), (F16, 18), (F16, 12)])
+def test_split_kernel(dims, nrhs, prec, reals):
+    kappa = 0.12
+    U = S.gauge_field(dims, 0.3, 31)
+    phi = np.stack([S.gaussian_spinor(dims, 80 + r) for r in range(nrhs)])
+    with Context(dims) as ctx:
+        ctx.gauge_upload(U, reals, prec)
+        H = gpu_hopping_full(ctx, phi if nrhs > 1 else phi[0], prec, nrhs).reshape(phi.shape)
+        for r in range(nrhs):
+            assert rel(H[r], C.hopping(U, phi[r])) <= TOL[prec]
+        if nrhs == 1:  # epilogues, both signs of the projectors
+            full, out = ctx.to_device(phi[0], prec), ctx.empty_full(prec)
+            ctx.twisted_apply(out, full, kappa, 0.3, prec)
+            g5 = np.array([1.0, 1, -1, -1])[:, None]
+            want = phi[0] - kappa * C.hopping(U, phi[0]) + 2j * kappa * 0.3 * g5 * phi[0]
+            assert rel(ctx.to_host(out, prec), want) <= TOL[prec]
+            e_in, e_out, tmp = ctx.halves(full, prec)[0], ctx.halves(out, prec)[0], ctx.empty_half(prec)
+            t, z, y, x = np.indices(phi.shape[1:5])
+            even = ((t + x + y + z) % 2 == 0)[..., None, None]
+            for dagger in (False, True):
+                ctx.schur_apply(e_out, e_in, tmp, kappa, prec, dagger=dagger)
+                v = np.where(even, g5 * phi[0] if dagger else phi[0], 0)
+                w = v - kappa**2 * C.hopping(U, C.hopping(U, v))
+                got = ctx.to_host(out, prec)[even[..., 0, 0]]
+                assert rel(got, (g5 * w if dagger else w)[even[..., 0, 0]]) <= TOL[prec]
