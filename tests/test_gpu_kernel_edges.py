@@ -128,3 +128,14 @@ def test_split_kernel(dims, nrhs, prec, reals):
                 w = v - kappa**2 * C.hopping(U, C.hopping(U, v))
                 got = ctx.to_host(out, prec)[even[..., 0, 0]]
                 assert rel(got, (g5 * w if dagger else w)[even[..., 0, 0]]) <= TOL[prec]
+
+
+def test_calls_follow_the_current_stream():
+    """Calls without a stream go to torch's current stream of the current device."""
+    side = torch.cuda.Stream()
+    assert plq._stream(None) == torch.cuda.current_stream().cuda_stream
+    for _ in range(2):
+        with torch.cuda.stream(side):
+            assert plq._stream(None) == side.cuda_stream == torch.cuda.current_stream().cuda_stream
+        assert plq._stream(None) == torch.cuda.current_stream().cuda_stream
+    assert plq._stream(side) == side.cuda_stream and plq._stream(5) == 5
