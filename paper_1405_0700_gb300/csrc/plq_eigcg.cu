@@ -591,15 +591,13 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, p, EPI_PLAIN, 0, nullptr, 0.0, FIN_NONE, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, mp, to, EPI_XPAY_NORM, 0, p, -kk, FIN_CG_ALPHA, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, mp, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true));
-                PLQ_TRY(hop(G.S, PLQ_F64, 0, q, to, EPI_XPAY, 1, mp, -kk, FIN_NONE, nullptr, true));
-                Reduce rb = reduce_of(c, FIN_CG_BETA);
-                PLQ_TRY(blas_cg_update(G.S.N, 1, xe, r, p, q, PLQ_F64, rb, c->state, s));
+                PLQ_TRY(hop(G.S, PLQ_F64, 0, r, to, EPI_XPAY_RUPD, 1, mp, -kk, FIN_CG_BETA, r, true));
                 if (eig) {  // raw r_{j+1} into its (FP32) slot of the search space
                     to32_kernel<<<grid_of(G.N, false), 256, 0, s>>>(G.N, Vb + (size_t)(vs + i) * E->slot,
                                                                     static_cast<const double2 *>(r), vscale);
                     PLQ_CUDA(cudaGetLastError());
                 }
-                return blas_cg_direction(G.S.N, 1, p, r, PLQ_F64, c->state, s);
+                return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s);
             };
             // one graph of exactly L iterations (the ones that fill V)
             cudaGraph_t graph = nullptr;

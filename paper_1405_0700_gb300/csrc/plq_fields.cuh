@@ -320,8 +320,11 @@ __device__ __forceinline__ bool finite2(double2 a) { return isfinite(a.x) && isf
 __device__ __forceinline__ void finalize_one(int fin, SolverState *state, const double *tot) {
     SolverState z = *state, *st = &z;
     // A frozen right-hand side contributed nothing to this reduction: its
-    // scalars must not change.
-    if (st->stop) return;
+    // scalars must not change (its last update of x and p has been made).
+    if (st->stop) {
+        if (fin == FIN_CG_ALPHA) state->xpend = 0;
+        return;
+    }
     switch (fin) {
     case FIN_CG_ALPHA:
         st->pAp = tot[0];
@@ -335,6 +338,7 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *state, const 
         st->beta = tot[0] / st->rho;
         st->beta32 = (float)st->beta;
         st->rho = tot[0];
+        st->xpend = 1;
         if (st->hist && st->iter < st->hist_cap) {
             st->hist[3 * st->iter + 1] = st->beta;
             st->hist[3 * st->iter + 2] = tot[0];
@@ -589,6 +593,13 @@ __device__ __forceinline__ bool all_frozen(const SolverState *st, int n) {
     bool f = true;
     for (int r = 0; r < n; ++r) f = f && st[r].stop;
     return f;
+}
+// The same, with what the finalize step does for frozen right-hand sides.
+__device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const Reduce &red) {
+    if (!all_frozen(st, n)) return false;
+    if (red.fin == FIN_CG_ALPHA && red.st && blockIdx.x == 0)
+        for (int r = ltid(); r < n; r += lsize()) red.st[r].xpend = 0;
+    return true;
 }
 
 // ---------------------------------------------------------------- geometry

@@ -385,6 +385,72 @@ __device__ __forceinline__ void hop_dir(const HopArgs &a, const SiteGeom &g, int
     hop_dir<P, R, MU, DAG, TBL, 1>(a, g, i, rr, a1);
 }
 
+// Sums of an epilogue.
+constexpr int epi_sums(int epi) {
+    return epi == EPI_XPAY_NORM || epi == EPI_XPAY_RUPD ? 1 : epi == EPI_XPAY_DOTW ? 2 : epi == EPI_XPAY_TS ? 3 : 0;
+}
+
+// alpha of a state in the arithmetic of the kernel
+template <class T>
+__device__ __forceinline__ T hop_alpha(const SolverState &st) {
+    if constexpr (sizeof(T) == 4) return st.alpha32;
+    else return st.alpha;
+}
+
+// Epilogue of one output site and right-hand side rr: acc holds H in on entry
+// and the output on return; EPI's sums over it go to column `t` of racc.
+template <int P, int EPI, int NVM, int RT>
+__device__ __forceinline__ void hop_epilogue(const HopArgs &a, size_t stride, long long idx, int rr, cx<RealOf<P>> acc[12],
+                                             RedAcc<NVM, RT> &racc, int t) {
+    using T = RealOf<P>;
+    if (a.twist_h) twist12(acc, hop_nu_h<T>(a), hop_scale_h<T>(a));
+    if constexpr (EPI != EPI_PLAIN) {
+        cx<T> xv[12];
+        Spinor<P>::load(a.x, stride, (size_t)idx, xv);
+        if (a.twist_x) twist12(xv, hop_nu_x<T>(a), T(1));
+        const T s = hop_a<T>(a);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            acc[k].re = fma(s, acc[k].re, xv[k].re);
+            acc[k].im = fma(s, acc[k].im, xv[k].im);
+        }
+        if constexpr (EPI == EPI_XPAY_RUPD) {
+            const T al = -hop_alpha<T>(a.st[rr]);
+            Spinor<P>::load(a.w, stride, (size_t)idx, xv);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) acc[k] = {fma(al, acc[k].re, xv[k].re), fma(al, acc[k].im, xv[k].im)};
+        }
+        if constexpr (EPI == EPI_XPAY_NORM || EPI == EPI_XPAY_RUPD) {
+            T s0 = 0;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) s0 = fma(acc[k].re, acc[k].re, fma(acc[k].im, acc[k].im, s0));
+            racc.add(0, t, s0);
+        } else if constexpr (EPI == EPI_XPAY_DOTW) {
+            cx<T> wv[12];
+            Spinor<P>::load(a.w, stride, (size_t)idx, wv);
+            T s0 = 0, s1 = 0;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {  // <w, out> = sum conj(w) out
+                s0 = fma(wv[k].re, acc[k].re, fma(wv[k].im, acc[k].im, s0));
+                s1 = fma(wv[k].re, acc[k].im, fma(-wv[k].im, acc[k].re, s1));
+            }
+            racc.add(0, t, s0);
+            racc.add(1, t, s1);
+        } else if constexpr (EPI == EPI_XPAY_TS) {
+            T s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {  // <out, x> and |out|^2
+                s0 = fma(acc[k].re, xv[k].re, fma(acc[k].im, xv[k].im, s0));
+                s1 = fma(acc[k].re, xv[k].im, fma(-acc[k].im, xv[k].re, s1));
+                s2 = fma(acc[k].re, acc[k].re, fma(acc[k].im, acc[k].im, s2));
+            }
+            racc.add(0, t, s0);
+            racc.add(1, t, s1);
+            racc.add(2, t, s2);
+        }
+    }
+}
+
 // Threads are arranged as (n / RT right-hand-side tiles) x (sites): the
 // threads of one site are adjacent and share its link loads through L1, and
 // each thread applies every link it loads to RT right-hand sides.
@@ -394,9 +460,9 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
     const int n = a.nrhs;
     const long long total = (long long)a.lat.Vh * n;
     const size_t stride = (size_t)total;
-    constexpr int NV = EPI == EPI_XPAY_NORM ? 1 : EPI == EPI_XPAY_DOTW ? 2 : EPI == EPI_XPAY_TS ? 3 : 0;
+    constexpr int NV = epi_sums(EPI);
     if constexpr (NV > 0) {
-        if (a.st != nullptr && all_frozen(a.st, n)) return;
+        if (a.st != nullptr && frozen_exit(a.st, n, a.red)) return;
     }
     RedAcc<(NV > 0 ? NV : 1), RT> racc;
     red_init(racc);
@@ -439,46 +505,7 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
             const int rr = r0 + t;
             if (RT > 1 && a.st != nullptr && a.st[rr].stop) continue;
             const long long idx = PLQ_GUARD(a.kstatus, (long long)i * n + rr, (long long)stride);
-            if (a.twist_h) twist12(acc[t], hop_nu_h<T>(a), hop_scale_h<T>(a));
-            if constexpr (EPI != EPI_PLAIN) {
-                cx<T> xv[12];
-                Spinor<P>::load(a.x, stride, (size_t)idx, xv);
-                if (a.twist_x) twist12(xv, hop_nu_x<T>(a), T(1));
-                const T s = hop_a<T>(a);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    acc[t][k].re = fma(s, acc[t][k].re, xv[k].re);
-                    acc[t][k].im = fma(s, acc[t][k].im, xv[k].im);
-                }
-                if constexpr (EPI == EPI_XPAY_NORM) {
-                    T s0 = 0;
-#pragma unroll
-                    for (int k = 0; k < 12; ++k) s0 = fma(acc[t][k].re, acc[t][k].re, fma(acc[t][k].im, acc[t][k].im, s0));
-                    racc.add(0, t, s0);
-                } else if constexpr (EPI == EPI_XPAY_DOTW) {
-                    cx<T> wv[12];
-                    Spinor<P>::load(a.w, stride, (size_t)idx, wv);
-                    T s0 = 0, s1 = 0;
-#pragma unroll
-                    for (int k = 0; k < 12; ++k) {  // <w, out> = sum conj(w) out
-                        s0 = fma(wv[k].re, acc[t][k].re, fma(wv[k].im, acc[t][k].im, s0));
-                        s1 = fma(wv[k].re, acc[t][k].im, fma(-wv[k].im, acc[t][k].re, s1));
-                    }
-                    racc.add(0, t, s0);
-                    racc.add(1, t, s1);
-                } else if constexpr (EPI == EPI_XPAY_TS) {
-                    T s0 = 0, s1 = 0, s2 = 0;
-#pragma unroll
-                    for (int k = 0; k < 12; ++k) {  // <out, x> and |out|^2
-                        s0 = fma(acc[t][k].re, xv[k].re, fma(acc[t][k].im, xv[k].im, s0));
-                        s1 = fma(acc[t][k].re, xv[k].im, fma(-acc[t][k].im, xv[k].re, s1));
-                        s2 = fma(acc[t][k].re, acc[t][k].re, fma(acc[t][k].im, acc[t][k].im, s2));
-                    }
-                    racc.add(0, t, s0);
-                    racc.add(1, t, s1);
-                    racc.add(2, t, s2);
-                }
-            }
+            hop_epilogue<P, EPI>(a, stride, idx, rr, acc[t], racc, t);
             Spinor<P>::store(a.out, stride, (size_t)idx, acc[t]);
         }
     }
@@ -577,7 +604,7 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
     float *sN = reinterpret_cast<float *>(sP + (size_t)NB * NP * blockDim.x * blockDim.y);
     const int n = a.nrhs;
     const size_t stride = (size_t)a.lat.Vh * n;
-    constexpr int NV = EPI == EPI_XPAY_NORM ? 1 : 0;
+    constexpr int NV = epi_sums(EPI);
     RedAcc<1, RT> racc;
     red_init(racc);
     const Lattice &L = a.lat;
@@ -591,7 +618,7 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
     if (a.st != nullptr) {
         // every right-hand side frozen (a solver's iterations past convergence):
         // nothing to stage or compute
-        if (all_frozen(a.st, n)) return;
+        if (frozen_exit(a.st, n, a.red)) return;
     }
     for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         __syncthreads();  // the previous site block is done with the shared links
@@ -754,24 +781,7 @@ __global__ void __maxnreg__(RT == 1 ? 80 : 168) hop_mrhs_kernel(const HopArgs a)
             const int rr = r0 + t;
             if (a.st != nullptr && a.st[rr].stop) continue;
             const long long idx = PLQ_GUARD(a.kstatus, (long long)i * n + rr, (long long)stride);
-            if (a.twist_h) twist12(acc[t], hop_nu_h<T>(a), hop_scale_h<T>(a));
-            if constexpr (EPI != EPI_PLAIN) {
-                cx<T> xv[12];
-                Spinor<P>::load(a.x, stride, (size_t)idx, xv);
-                if (a.twist_x) twist12(xv, hop_nu_x<T>(a), T(1));
-                const T s = hop_a<T>(a);
-#pragma unroll
-                for (int e = 0; e < 12; ++e) {
-                    acc[t][e].re = fma(s, acc[t][e].re, xv[e].re);
-                    acc[t][e].im = fma(s, acc[t][e].im, xv[e].im);
-                }
-                if constexpr (EPI == EPI_XPAY_NORM) {
-                    T s0 = 0;
-#pragma unroll
-                    for (int e = 0; e < 12; ++e) s0 = fma(acc[t][e].re, acc[t][e].re, fma(acc[t][e].im, acc[t][e].im, s0));
-                    racc.add(0, t, s0);
-                }
-            }
+            hop_epilogue<P, EPI>(a, stride, idx, rr, acc[t], racc, t);
             Spinor<P>::store(a.out, stride, (size_t)idx, acc[t]);
         }
     }
@@ -833,6 +843,7 @@ plq_status dispatch_mrhs(const HopArgs &a, int epi, cudaStream_t s, int block) {
     case EPI_XPAY:
         return a.dagger ? launch_mrhs_t<P, R, EPI_XPAY, true, RT, NB>(a, s, block)
                         : launch_mrhs_t<P, R, EPI_XPAY, false, RT, NB>(a, s, block);
+    case EPI_XPAY_RUPD: return launch_mrhs_t<P, R, EPI_XPAY_RUPD, true, RT, NB>(a, s, block);
     default:
         return a.dagger ? launch_mrhs_t<P, R, EPI_XPAY_NORM, true, RT, NB>(a, s, block)
                         : launch_mrhs_t<P, R, EPI_XPAY_NORM, false, RT, NB>(a, s, block);
@@ -901,6 +912,7 @@ plq_status dispatch_tiled(const HopArgs &a, int epi, cudaStream_t s, int block) 
     case EPI_XPAY:
         return a.dagger ? launch_hop_t<P, R, EPI_XPAY, true, false, RT>(a, s, block)
                         : launch_hop_t<P, R, EPI_XPAY, false, false, RT>(a, s, block);
+    case EPI_XPAY_RUPD: return launch_hop_t<P, R, EPI_XPAY_RUPD, true, false, RT>(a, s, block);
     default:
         return a.dagger ? launch_hop_t<P, R, EPI_XPAY_NORM, true, false, RT>(a, s, block)
                         : launch_hop_t<P, R, EPI_XPAY_NORM, false, false, RT>(a, s, block);
@@ -928,16 +940,18 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
             return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
         }
     }
+    if (epi == EPI_XPAY_RUPD && !a.dagger) return set_error(PLQ_ERR_ARG, "the residual update belongs to the adjoint");
     if constexpr (P != PLQ_F64) {
+        const bool cg_epi = epi <= EPI_XPAY_NORM || epi == EPI_XPAY_RUPD;
         if (a.smem_links == 4 && a.site_begin == 0 && a.site_end < 0 && epi <= EPI_XPAY_NORM)
             return dispatch_rows<P, R>(a, epi, s);
-        if (a.smem_links && a.nrhs > 1 && a.site_begin == 0 && a.site_end < 0 && epi <= EPI_XPAY_NORM) {
+        if (a.smem_links && a.nrhs > 1 && a.site_begin == 0 && a.site_end < 0 && cg_epi) {
             if (a.rhs_tile == 2 && a.nrhs % 2 == 0) return dispatch_mrhs<P, R, 2, 0>(a, epi, s, block);
             if (a.smem_links == 2) return dispatch_mrhs<P, R, 1, 2>(a, epi, s, block);
             if (a.smem_links == 3) return dispatch_mrhs<P, R, 1, 3>(a, epi, s, block);
             return dispatch_mrhs<P, R, 1, 0>(a, epi, s, block);
         }
-        if (a.rhs_tile > 1 && a.nrhs % a.rhs_tile == 0 && epi <= EPI_XPAY_NORM) {
+        if (a.rhs_tile > 1 && a.nrhs % a.rhs_tile == 0 && cg_epi) {
             if (a.rhs_tile == 2) return dispatch_tiled<P, R, 2>(a, epi, s, block);
             if (a.rhs_tile == 4) return dispatch_tiled<P, R, 4>(a, epi, s, block);
         }
@@ -960,6 +974,9 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
                             : launch_hop_t<P, R, EPI_XPAY_NORM, false, true>(a, s, block);
         return a.dagger ? launch_hop_t<P, R, EPI_XPAY_NORM, true>(a, s, block)
                         : launch_hop_t<P, R, EPI_XPAY_NORM, false>(a, s, block);
+    case EPI_XPAY_RUPD:
+        if (tbl) return launch_hop_t<P, R, EPI_XPAY_RUPD, true, true>(a, s, block);
+        return launch_hop_t<P, R, EPI_XPAY_RUPD, true>(a, s, block);
     case EPI_XPAY_DOTW:
         return launch_hop_t<P, R, EPI_XPAY_DOTW, false>(a, s, block);
     case EPI_XPAY_TS:

@@ -157,9 +157,9 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
     using V = typename PL::V;
     __shared__ __align__(16) cx<T> part[8 * 6 * 32];  // (direction, upper component, element)
     __shared__ cx<T> res[P == PLQ_F16 ? 12 * 32 : 1];  // FP16 storage: the element's output until its norm is known
-    constexpr int NV = EPI == EPI_XPAY_NORM ? 1 : EPI == EPI_XPAY_DOTW ? 2 : EPI == EPI_XPAY_TS ? 3 : 0;
+    constexpr int NV = epi_sums(EPI);
     const int n = a.nrhs;
-    if (a.st != nullptr && all_frozen(a.st, n)) return;
+    if (a.st != nullptr && frozen_exit(a.st, n, a.red)) return;
     RedAcc<(NV > 0 ? NV : 1), 1> racc;
     red_init(racc);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -212,8 +212,14 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
                     const T s = hop_a<T>(a);
 #pragma unroll
                     for (int q = 0; q < PL::N; ++q) o[q] = {fma(s, o[q].re, x[q].re), fma(s, o[q].im, x[q].im)};
+                    if constexpr (EPI == EPI_XPAY_RUPD) {  // (one right-hand side)
+                        const T al = -hop_alpha<T>(a.st[0]);
+                        load_plane<P>(a.w, stride, (size_t)e, k, x);
+#pragma unroll
+                        for (int q = 0; q < PL::N; ++q) o[q] = {fma(al, o[q].re, x[q].re), fma(al, o[q].im, x[q].im)};
+                    }
                     T s0 = 0, s1 = 0, s2 = 0;
-                    if constexpr (EPI == EPI_XPAY_NORM) {
+                    if constexpr (EPI == EPI_XPAY_NORM || EPI == EPI_XPAY_RUPD) {
 #pragma unroll
                         for (int q = 0; q < PL::N; ++q) s0 = fma(o[q].re, o[q].re, fma(o[q].im, o[q].im, s0));
                     } else if constexpr (EPI == EPI_XPAY_DOTW) {
@@ -279,6 +285,9 @@ plq_status dispatch_split(const HopArgs &a, int epi, cudaStream_t s) {
     case EPI_XPAY: return a.dagger ? launch_split_t<P, R, EPI_XPAY, true>(a, s) : launch_split_t<P, R, EPI_XPAY, false>(a, s);
     case EPI_XPAY_NORM:
         return a.dagger ? launch_split_t<P, R, EPI_XPAY_NORM, true>(a, s) : launch_split_t<P, R, EPI_XPAY_NORM, false>(a, s);
+    case EPI_XPAY_RUPD:
+        if (!a.dagger) return set_error(PLQ_ERR_ARG, "the residual update belongs to the adjoint");
+        return launch_split_t<P, R, EPI_XPAY_RUPD, true>(a, s);
     case EPI_XPAY_DOTW: return launch_split_t<P, R, EPI_XPAY_DOTW, false>(a, s);
     case EPI_XPAY_TS: return launch_split_t<P, R, EPI_XPAY_TS, false>(a, s);
     default: return set_error(PLQ_ERR_ARG, "bad epilogue %d", epi);

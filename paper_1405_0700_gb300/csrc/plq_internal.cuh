@@ -110,7 +110,7 @@ struct SolverState {
     // |r_{j+1}|^2 for iteration j < hist_cap.
     double *hist;
     int hist_cap;
-    int pad2;
+    int xpend;        // CG: this iteration's x += alpha p (and p = r + beta p unless stopped) is due
     // The coefficients as FP32 kernels use them, converted once where they are
     // computed: a conversion costs every warp that makes it 15 cycles of the
     // FP64 pipe.
@@ -224,6 +224,9 @@ enum Epilogue {
     EPI_XPAY_NORM = 2,  // ... and sum |out|^2
     EPI_XPAY_DOTW = 3,  // ... and sum <w, out> (complex)
     EPI_XPAY_TS = 4,    // ... and sum <out, x> (complex), |out|^2
+    // q = x + a * H in, out = w - alpha q with alpha from the states, sum |out|^2: the
+    // residual update of CG (w may be out) without q's way through memory
+    EPI_XPAY_RUPD = 5,
 };
 
 struct HopArgs {
@@ -315,9 +318,8 @@ plq_status blas_gamma5(long long N, void *dst, const void *src, int prec, cudaSt
 plq_status blas_norm2(long long N, int n, const void *v, int prec, const Reduce &red, cudaStream_t s);
 plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int prec, const Reduce &red,
                          cudaStream_t s);
-// x += alpha p; r -= alpha q; rho_new = |r|^2
-plq_status blas_cg_update(long long N, int n, void *x, void *r, const void *p, const void *q, int prec,
-                          const Reduce &red, const SolverState *st, cudaStream_t s);
+// x += alpha p, then p = r + beta p unless the right-hand side has stopped; where xpend is set
+plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s);
 // p = r + beta p
 plq_status blas_cg_direction(long long N, int n, void *p, const void *r, int prec, const SolverState *st,
                              cudaStream_t s);

@@ -151,7 +151,7 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
     const size_t h64 = spinor_site_bytes(PLQ_F64) * (size_t)S.N;
     const size_t hL = spinor_site_bytes(S.P) * (size_t)S.N;
     const size_t hX = spinor_site_bytes(S.PX) * (size_t)S.N;
-    const int nL = method == SOLVER_CG ? 5 : 7;
+    const int nL = method == SOLVER_CG ? 4 : 7;
     const size_t need = 5 * h64 + nL * hL + hX + 4096;
     PLQ_TRY(ensure_work(c, need));
     char *w = static_cast<char *>(c->work);
@@ -322,7 +322,7 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                 // FP64 true residual; r only restarts the inner iteration, so with
                 // a low-precision inner solve it is formed at that precision (two
                 // inner-precision half-applies instead of two FP64 ones).
-                void *rL = L[0], *pL = L[1], *qL = L[2], *mpL = L[3], *toL = L[4];
+                void *rL = L[0], *pL = L[1], *mpL = L[2], *toL = L[3];
                 if (S.P == PLQ_F64) {
                     if ((st = hop(S, PLQ_F64, 1, tmp_o64, s64, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, false,
                                   tw_first(S, true))) != PLQ_OK)
@@ -368,10 +368,9 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     PLQ_TRY(hop(S, PI, 0, mpL, toL, EPI_XPAY_NORM, 0, pL, -kk, FIN_CG_ALPHA, nullptr, true,
                                 tw_second(S, false)));
                     PLQ_TRY(hop(S, PI, 1, toL, mpL, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true, tw_first(S, true)));
-                    PLQ_TRY(hop(S, PI, 0, qL, toL, EPI_XPAY, 1, mpL, -kk, FIN_NONE, nullptr, true, tw_second(S, true)));
-                    Reduce rb = reduce_of(c, FIN_CG_BETA);
-                    PLQ_TRY(blas_cg_update(S.N, n, xL, rL, pL, qL, PI, rb, c->state, s));
-                    return blas_cg_direction(S.N, n, pL, rL, PI, c->state, s);
+                    // r -= alpha Mhat^dagger Mhat p, |r|^2; then x += alpha p, p = r + beta p
+                    PLQ_TRY(hop(S, PI, 0, rL, toL, EPI_XPAY_RUPD, 1, mpL, -kk, FIN_CG_BETA, rL, true, tw_second(S, true)));
+                    return blas_cg_xp(S.N, n, xL, pL, rL, PI, c->state, s);
                 };
                 if ((st = run_batches(S, P.k, body, fin, &c->solve_graph[method], gkey)) != PLQ_OK) break;
             } else {
