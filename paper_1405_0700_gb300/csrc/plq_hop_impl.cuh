@@ -940,6 +940,23 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
             return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
         }
     }
+    if constexpr (P != PLQ_F64) {
+        // Links staged in shared memory or read by every right-hand side's thread:
+        // staging costs two barriers per block and pays once enough right-hand sides
+        // share a link.  FP32, direct / staged (blocks of 96): 24^3x48 12-real 9 RHS
+        // 206 / 222 us, 11 RHS 259 / 249, 12 RHS 274 / 236; 32^3x64 10 RHS 792 / 810,
+        // 11 RHS 898 / 830; 48^3x96 12 RHS 5683 / 4306, 18-real 5277 / 4457 (32^3x64
+        // 18-real 12 RHS 842 / 865 is the exception).  FP16, direct / staged (128):
+        // 24^3x48 12-real 3 RHS 76 / 78, 5 RHS 122 / 115, 9 RHS 219 / 191, 12 RHS
+        // 317 / 247; 32^3x64 18-real 5 RHS 375 / 379, 9 RHS 677 / 642.
+        if (a.untuned && a.nrhs >= (P == PLQ_F16 ? 5 : 11)) {
+            HopArgs d = a;
+            d.untuned = 0;
+            d.smem_links = 1;
+            d.block = P == PLQ_F16 ? 128 : 96;
+            return dispatch_hop<P, R>(d, epi, s, d.block);
+        }
+    }
     if (epi == EPI_XPAY_RUPD && !a.dagger) return set_error(PLQ_ERR_ARG, "the residual update belongs to the adjoint");
     if constexpr (P != PLQ_F64) {
         const bool cg_epi = epi <= EPI_XPAY_NORM || epi == EPI_XPAY_RUPD;
