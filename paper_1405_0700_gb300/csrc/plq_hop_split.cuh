@@ -218,7 +218,11 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
 #pragma unroll
                         for (int q = 0; q < PL::N; ++q) o[q] = {fma(al, o[q].re, x[q].re), fma(al, o[q].im, x[q].im)};
                     }
-                    T s0 = 0, s1 = 0, s2 = 0;
+                    // (FP64 sums go on in the thread's accumulators, whose additions the
+                    // fused multiply-adds then are; FP32 ones are added in FP64)
+                    constexpr bool go_on = NV > 0 && sizeof(T) == 8;
+                    T s0 = go_on ? (T)racc.v[0][0] : T(0), s1 = go_on && NV > 1 ? (T)racc.v[NV > 1 ? 1 : 0][0] : T(0),
+                      s2 = go_on && NV > 2 ? (T)racc.v[NV > 2 ? 2 : 0][0] : T(0);
                     if constexpr (EPI == EPI_XPAY_NORM || EPI == EPI_XPAY_RUPD) {
 #pragma unroll
                         for (int q = 0; q < PL::N; ++q) s0 = fma(o[q].re, o[q].re, fma(o[q].im, o[q].im, s0));
@@ -238,9 +242,9 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
                             s2 = fma(o[q].re, o[q].re, fma(o[q].im, o[q].im, s2));
                         }
                     }
-                    if constexpr (NV >= 1) racc.add(0, 0, s0);
-                    if constexpr (NV >= 2) racc.add(1, 0, s1);
-                    if constexpr (NV >= 3) racc.add(2, 0, s2);
+                    const T sums[3] = {s0, s1, s2};
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) racc.v[q][0] = go_on ? (double)sums[q] : racc.v[q][0] + (double)sums[q];
                 }
                 if constexpr (P == PLQ_F16) {
                     res[(2 * k) * 32 + lane] = o[0];
