@@ -128,7 +128,8 @@ typedef struct {
                           default 1e-4 for FP32 (1e-3 for BiCGstab), 1e-2 for FP16 inner
                           solves (ignored when inner_prec == PLQ_F64)                       */
     int use_x0;        /* 1: x holds an initial guess on entry (resume); 0: start from 0   */
-    int check_every;   /* inner iterations per host convergence poll, default 16           */
+    int check_every;   /* accepted and not used: the device ends its iterations by itself,
+                          without polls of the host                                       */
     double mu;         /* twisted mass: solve M_tm = 1 - kappa H + 2 i kappa mu gamma5
                           (0: the Wilson operator M)                                        */
     int residual_prec; /* arithmetic of the FP64-accuracy steps of a mixed-precision solve

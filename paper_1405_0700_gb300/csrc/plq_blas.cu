@@ -324,7 +324,7 @@ __global__ void bicg_update_kernel(long long N, int n, void *x, void *r, const v
                                    const void *t, const void *rhat, Reduce red, const SolverState *st) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
-    if (all_frozen(st, n)) return;
+    if (frozen_exit(st, n, red)) return;
     RedAcc<3> acc;
     red_init(acc);
     ELEM_LOOP(N) {

@@ -426,6 +426,24 @@ __device__ __forceinline__ V warp_sum(V x, int lane, int active) {
     return x;
 }
 
+// Every one of n right-hand sides frozen.  A reducing kernel may then leave at
+// once, without its ticket: states change only in the finalize step of a last
+// block, after every block of that launch has read them here, so all blocks of
+// a launch decide alike.
+__device__ __forceinline__ bool all_frozen(const SolverState *st, int n) {
+    bool f = true;
+    for (int r = 0; r < n; ++r) f = f && st[r].stop;
+    return f;
+}
+// The same, with what the finalize step does for frozen right-hand sides.
+__device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const Reduce &red) {
+    if (!all_frozen(st, n)) return false;
+    if (red.fin == FIN_CG_ALPHA && red.st && blockIdx.x == 0)
+        for (int r = ltid(); r < n; r += lsize()) red.st[r].xpend = 0;
+    if (red.cond && blockIdx.x == 0 && ltid() == 0) cudaGraphSetConditional(red.cond, 0);
+    return true;
+}
+
 // Block sums of the RedAcc values: total (value v, column c) goes to
 // slot[(k*n + c*RT) + t], v = k*RT + t, valid for every thread after the
 // closing barrier.  wv: kRedThreads * W doubles (W <= 4) or 32 * (warps) (W = 32).
@@ -521,7 +539,7 @@ __device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols
 // slot group are in flight together.  Measured (with the early exit of
 // all_frozen and the FP32 coefficients of SolverState): mixed BiCGstab on
 // 20x12x28x36 8.10 -> 5.46 ms, EigCG on 16^3x32 303 -> 272 ms (its 32-value
-// sums 234 -> 130 us), FP64 norm of a 24^3x48 half field 35 -> 25 us.
+// sums 234 -> 92 us), FP64 norm of a 24^3x48 half field 35 -> 25 us.
 template <int NV, int RT>
 __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int ncols) {
     constexpr int W = NV * RT;
@@ -581,25 +599,12 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int nc
             for (int k = 0; k < NV; ++k) tr[k] = slot[k * n + r];
             finalize_one(red.fin, red.st + r, tr);
         }
+        if (red.cond) {
+            __syncthreads();
+            if (tid == 0 && all_frozen(red.st, n)) cudaGraphSetConditional(red.cond, 0);
+        }
     }
     if (tid == 0) *red.ticket = 0u;
-}
-
-// Every one of n right-hand sides frozen.  A reducing kernel may then leave at
-// once, without its ticket: states change only in the finalize step of a last
-// block, after every block of that launch has read them here, so all blocks of
-// a launch decide alike.
-__device__ __forceinline__ bool all_frozen(const SolverState *st, int n) {
-    bool f = true;
-    for (int r = 0; r < n; ++r) f = f && st[r].stop;
-    return f;
-}
-// The same, with what the finalize step does for frozen right-hand sides.
-__device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const Reduce &red) {
-    if (!all_frozen(st, n)) return false;
-    if (red.fin == FIN_CG_ALPHA && red.st && blockIdx.x == 0)
-        for (int r = ltid(); r < n; r += lsize()) red.st[r].xpend = 0;
-    return true;
 }
 
 // ---------------------------------------------------------------- geometry

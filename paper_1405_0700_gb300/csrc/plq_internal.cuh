@@ -137,6 +137,9 @@ struct Reduce {
     double *sums = nullptr;       // grid totals: sums[k * nrhs + r]
     SolverState *st = nullptr;    // per right-hand side targets of the finalize step (array of nrhs)
     int fin = FIN_NONE;
+    // the loop this launch ends an iteration of (a conditional graph node): the
+    // launch ends the loop once every state has stopped; 0: no loop
+    unsigned long long cond = 0;
 };
 
 constexpr int kMaxReduceBlocks = 4096;
@@ -177,10 +180,10 @@ struct Ctx {
     cudaStream_t copy_in = nullptr, copy_out = nullptr, compute = nullptr;  // host-path pipeline
     cudaEvent_t ev[3 * 64] = {};
     int num_sms = 0;
-    // Instantiated inner-iteration graph of the last CG / BiCGstab solve, reused
+    // Instantiated inner-iteration loop of the last CG / BiCGstab solve, reused
     // by the next reliable-update cycle and the next solve with the same key
-    // (method, precisions, sizes, kappa, mu, batch length, workspace address,
-    // launch configuration version, inner gauge copy address and format).
+    // (method, precisions, sizes, kappa, mu, workspace address, launch
+    // configuration version, inner gauge copy address and format).
     struct SolveGraph {
         cudaGraphExec_t exec = nullptr;
         unsigned long long key[10] = {};

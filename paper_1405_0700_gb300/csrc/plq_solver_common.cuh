@@ -1,6 +1,6 @@
 // Host-side helpers shared by the solver translation units: the launch of
 // one hopping half-application inside a solve, reductions read back to the
-// host, device solver states and graph-captured batches of iterations.
+// host, device solver states and the graph-captured loop of iterations.
 #pragma once
 
 #include <cstring>
@@ -22,6 +22,7 @@ struct Solve {
     int PX;  // inner solution accumulator precision
     double nu = 0.0;  // twisted mass: nu = 2 kappa mu (0 = Wilson)
     double hops = 0;
+    cudaGraphConditionalHandle loop = 0;  // of the loop whose body is being captured
 };
 
 // Twisted-mass terms of one hopping launch (all zero / one for Wilson).
@@ -56,6 +57,7 @@ plq_status hop(Solve &S, int prec, int out_par, void *out, const void *in, int e
     h.lat = c->lat;
     h.red = reduce_of(c, fin);
     if (fin == FIN_NONE) h.red.st = nullptr;
+    if (fin == FIN_CG_BETA) h.red.cond = S.loop;
     h.st = freeze ? c->state : nullptr;
     h.nu_x = tw.nu_x;
     h.nu_h = tw.nu_h;
@@ -113,67 +115,61 @@ plq_status get_states(Solve &S, std::vector<SolverState> &st) {
     return PLQ_OK;
 }
 
-// Run `body` (one inner iteration) as graph-captured batches of `k` until the
-// device state of every right-hand side says stop.  With a cache, the
-// instantiated graph is kept and reused while the key matches (the body's
-// launches depend only on what the key records).
+// Run `body` (one inner iteration) on the device until the state of every
+// right-hand side says stop: the body is captured once into a while node of a
+// graph, whose last reduction of an iteration ends the loop.  (Every pass either
+// advances `iter` of a right-hand side that has not stopped, up to maxit, or
+// finds all stopped, so the loop ends.)  The instantiated graph is kept in
+// `cache` and reused while the key matches; the launches depend only on what
+// the key records.
+//
+// Batches of 16 captured iterations with a poll of the host after each ran 8
+// iterations too many per reliable-update cycle, launches that find everything
+// frozen and leave: mixed BiCGstab on 20x12x28x36 (53 of its 80 iterations) 5.37
+// -> 4.77 ms, mixed CG on 8^3x16 2.40 -> 2.18 ms, on 24^3x48 no change.  A pass
+// of the loop costs a few us beside its launches; one to six iterations per pass:
+// CG on 24^3x48 16.25, 16.11, 16.06, 16.08, 16.09 ms (1, 2, 3, 4, 6), CG on 8^3x16
+// 2.31, 2.22, 2.18, 2.20, 2.19 ms, BiCGstab 4.84, 4.87, 4.86, 4.91, 4.93 ms.
+constexpr int kLoopBody = 3;
+
 template <class Body>
-plq_status run_batches(Solve &S, int k, Body body, std::vector<SolverState> &cur, Ctx::SolveGraph *cache = nullptr,
-                       const unsigned long long *key = nullptr) {
-    cudaGraphExec_t exec = nullptr;
-    plq_status st = PLQ_OK;
-    cudaError_t e = cudaSuccess;
-    if (cache && cache->exec && std::memcmp(cache->key, key, sizeof(cache->key)) == 0) {
-        exec = cache->exec;
-    } else {
-        cudaGraph_t graph = nullptr;
-        PLQ_CUDA(cudaStreamBeginCapture(S.s, cudaStreamCaptureModeThreadLocal));
-        const double hops0 = S.hops;
-        for (int i = 0; i < k && st == PLQ_OK; ++i) st = body();
-        e = cudaStreamEndCapture(S.s, &graph);
-        S.hops = hops0;
-        if (st != PLQ_OK) {
-            if (graph) cudaGraphDestroy(graph);
-            return st;
+plq_status run_loop(Solve &S, Body body, std::vector<SolverState> &cur, Ctx::SolveGraph &cache, const unsigned long long *key) {
+    if (!(cache.exec && std::memcmp(cache.key, key, sizeof(cache.key)) == 0)) {
+        cudaGraph_t graph = nullptr, captured = nullptr;
+        PLQ_CUDA(cudaGraphCreate(&graph, 0));
+        cudaGraphNode_t node = nullptr;
+        cudaGraphNodeParams np{};
+        np.type = cudaGraphNodeTypeConditional;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaError_t e = cudaGraphConditionalHandleCreate(&np.conditional.handle, graph, 1, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
+        plq_status st = PLQ_OK;
+        if (e == cudaSuccess)
+            e = cudaStreamBeginCaptureToGraph(S.s, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                              cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            const double hops0 = S.hops;
+            S.loop = np.conditional.handle;
+            for (int i = 0; i < kLoopBody && st == PLQ_OK; ++i) st = body();
+            S.loop = 0;
+            S.hops = hops0;
+            e = cudaStreamEndCapture(S.s, &captured);
         }
-        if (e != cudaSuccess) return cuda_error(e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&exec, graph, 0);
+        cudaGraphExec_t exec = nullptr;
+        if (st == PLQ_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
-        if (e != cudaSuccess) return cuda_error(e, "cudaGraphInstantiate");
-        if (cache) {
-            if (cache->exec) cudaGraphExecDestroy(cache->exec);
-            cache->exec = exec;
-            std::memcpy(cache->key, key, sizeof(cache->key));
-        }
+        if (st != PLQ_OK) return st;
+        if (e != cudaSuccess) return cuda_error(e, "solver iteration graph");
+        if (cache.exec) cudaGraphExecDestroy(cache.exec);
+        cache.exec = exec;
+        std::memcpy(cache.key, key, sizeof(cache.key));
     }
-    long long last_sum = -1;
-    int idle = 0;
-    for (;;) {
-        e = cudaGraphLaunch(exec, S.s);
-        if (e != cudaSuccess) {
-            st = cuda_error(e, "cudaGraphLaunch");
-            break;
-        }
-        st = get_states(S, cur);
-        if (st != PLQ_OK) break;
-        bool all = true;
-        long long sum = 0;
-        for (int r = 0; r < S.n; ++r) {
-            all = all && cur[r].stop;
-            sum += cur[r].iter;
-        }
-        if (all) break;
-        // every batch advances some right-hand side unless all are frozen; a
-        // state that neither advances nor stops is a logic error, not a hang
-        idle = (sum == last_sum) ? idle + 1 : 0;
-        last_sum = sum;
-        if (idle >= 2) {
-            st = set_error(PLQ_ERR_STATE, "inner iteration made no progress");
-            break;
-        }
-    }
-    if (!cache) cudaGraphExecDestroy(exec);
-    return st;
+    PLQ_CUDA(cudaGraphLaunch(cache.exec, S.s));
+    PLQ_TRY(get_states(S, cur));
+    for (int r = 0; r < S.n; ++r)
+        if (!cur[r].stop) return set_error(PLQ_ERR_STATE, "inner iteration ended before right-hand side %d stopped", r);
+    return PLQ_OK;
 }
 
 }  // namespace

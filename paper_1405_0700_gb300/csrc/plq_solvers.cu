@@ -24,9 +24,9 @@
 //
 // Each inner iteration is a fixed sequence of kernels that read their
 // coefficients from device-resident SolverStates and update them in the last
-// block of each fused reduction; a batch of `check_every` iterations is
-// captured once into a CUDA graph and replayed, and the host only polls the
-// states between batches.  Once a right-hand side's stop flag is set
+// block of each fused reduction; it is captured once as the body of a while
+// node of a CUDA graph, which runs until every right-hand side has stopped
+// without the host.  Once a right-hand side's stop flag is set
 // (triggered, converged, maxit, NaN or breakdown) every later kernel skips its
 // elements, so its x and r stay consistent.
 #include <chrono>
@@ -46,7 +46,6 @@ struct Params {
     int inner;
     double delta;
     int use_x0;
-    int k;
     double mu;
     int residual;  // PLQ_F64 or PLQ_DF64 arithmetic of the reliable-update residuals
 };
@@ -64,12 +63,10 @@ plq_status parse(const plq_solver_params *p, Params *o) {
     const int inner = p ? p->inner_prec : PLQ_F64;
     o->delta = (p && p->delta > 0) ? p->delta : (inner == PLQ_F16 ? 1e-2 : 1e-4);
     o->use_x0 = p ? p->use_x0 : 0;
-    o->k = (p && p->check_every > 0) ? p->check_every : 16;
     o->mu = p ? p->mu : 0.0;
     if (!std::isfinite(o->mu)) return set_error(PLQ_ERR_ARG, "twisted mass mu not finite");
     if (!valid_prec(o->inner)) return set_error(PLQ_ERR_ARG, "bad inner precision %d", o->inner);
     if (o->delta >= 1.0) return set_error(PLQ_ERR_ARG, "delta must be < 1");
-    if (o->k > 256) o->k = 256;
     o->residual = p ? p->residual_prec : PLQ_F64;
     if (o->residual != PLQ_F64 && o->residual != PLQ_DF64)
         return set_error(PLQ_ERR_ARG, "residual_prec must be PLQ_F64 or PLQ_DF64");
@@ -169,7 +166,6 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
         gkey[2] = (unsigned long long)S.N;
         std::memcpy(&gkey[3], &kk, sizeof(double));
         std::memcpy(&gkey[4], &nu, sizeof(double));
-        gkey[5] = (unsigned long long)P.k;
         gkey[6] = (unsigned long long)reinterpret_cast<uintptr_t>(c->work);
         gkey[7] = (unsigned long long)c->tune_version;
         gkey[8] = 1;  // marks a valid key
@@ -372,7 +368,7 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     PLQ_TRY(hop(S, PI, 0, rL, toL, EPI_XPAY_RUPD, 1, mpL, -kk, FIN_CG_BETA, rL, true, tw_second(S, true)));
                     return blas_cg_xp(S.N, n, xL, pL, rL, PI, c->state, s);
                 };
-                if ((st = run_batches(S, P.k, body, fin, &c->solve_graph[method], gkey)) != PLQ_OK) break;
+                if ((st = run_loop(S, body, fin, c->solve_graph[method], gkey)) != PLQ_OK) break;
             } else {
                 void *rL = L[0], *rhL = L[1], *pL = L[2], *vL = L[3], *sL = L[4], *tL = L[5], *toL = L[6];
                 if ((st = blas_scale64(S.N, n, s64, sc.data(), s)) != PLQ_OK) break;
@@ -400,10 +396,11 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     PLQ_TRY(hop(S, PI, 0, tL, toL, EPI_XPAY_TS, 0, sL, -kk, FIN_BICG_OMEGA, nullptr, true,
                                 tw_second(S, false)));
                     Reduce rb = reduce_of(c, FIN_BICG_RHO);
+                    rb.cond = S.loop;
                     PLQ_TRY(blas_bicg_update(S.N, n, xL, rL, pL, sL, tL, rhL, PI, rb, c->state, s));
                     return blas_bicg_p(S.N, n, pL, rL, vL, PI, c->state, s);
                 };
-                if ((st = run_batches(S, P.k, body, fin, &c->solve_graph[method], gkey)) != PLQ_OK) break;
+                if ((st = run_loop(S, body, fin, c->solve_graph[method], gkey)) != PLQ_OK) break;
             }
             for (int r = 0; r < n; ++r) {
                 if (done[r]) continue;
