@@ -387,7 +387,8 @@ typedef struct {
  * rewriting the descriptors, so it may solve other systems, sources or
  * kappas.  The launch shape (threads per block, resident blocks per SM) is
  * the one set on ctxs[0] by plq_set_batched_launch or plq_autotune_batched,
- * else 128 threads and all blocks that fit.
+ * else 192 threads (lattices of 800,000 sites or more in all) or 128, and all
+ * blocks that fit.
  *
  * Batched CG: n (1..64) independent systems M_k x_k = b_k -- different
  * lattices (one context each, same device), kappas and iteration counts --

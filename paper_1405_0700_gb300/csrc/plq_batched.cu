@@ -12,6 +12,16 @@
 using namespace plq;
 using namespace plq::batch;
 
+namespace {
+
+int shape_of_block(int block) {
+    for (int k = 0; k < kNumShapes; ++k)
+        if (kShapes[k].block == block) return k;
+    return -1;
+}
+
+}  // namespace
+
 extern "C" plq_status plq_cg_solve_batched(plq_ctx **ctxs, int n, void **x, const void **b, const double *kappa,
                                            const plq_solver_params *params, plq_solve_info *infos,
                                            plq_batch_info *binfo, void *stream) {
@@ -54,7 +64,7 @@ extern "C" plq_status plq_cg_solve_batched(plq_ctx **ctxs, int n, void **x, cons
         const size_t Vh = c->lat.Vh;
         const size_t h64 = spinor_site_bytes(PLQ_F64) * Vh, hL = spinor_site_bytes(inner) * Vh,
                      hX = spinor_site_bytes(PX) * Vh;
-        PLQ_TRY(ensure_work(c, 3 * h64 + 5 * hL + hX + 4096));
+        PLQ_TRY(ensure_work(c, 3 * h64 + 4 * hL + hX + 4096));
         char *w = static_cast<char *>(c->work);
         BatchSystem &B = sys[k];
         B.lat = c->lat;
@@ -78,10 +88,9 @@ extern "C" plq_status plq_cg_solve_batched(plq_ctx **ctxs, int n, void **x, cons
         char *wl = w + 3 * h64;
         B.rL = wl;
         B.pL = wl + hL;
-        B.qL = wl + 2 * hL;
-        B.mpL = wl + 3 * hL;
-        B.toL = wl + 4 * hL;
-        B.xL = wl + 5 * hL;
+        B.mpL = wl + 2 * hL;
+        B.toL = wl + 3 * hL;
+        B.xL = wl + 4 * hL;
     }
     // small batch scratch: descriptors, results, accumulators, barrier words;
     // kept in the first context with its stream and instantiated graph
@@ -140,11 +149,19 @@ extern "C" plq_status plq_cg_solve_batched(plq_ctx **ctxs, int n, void **x, cons
             stt = set_error(PLQ_ERR_ARG, "FP16 inner solves use 12-real links");
             break;
         }
+        // Launch shape until one is set or tuned: blocks of 192 threads with 168
+        // registers, which spill little, for batches of many sites (16 systems,
+        // 2.0 M sites: 92.9 against 96.8 ms with 128 threads; 6 FP16 systems, 0.8 M:
+        // 52.3 / 54.4 ms), 128 threads for the others, whose phases are short (4
+        // systems, 0.14 M: 11.17 / 11.00 ms).
+        long long sites = 0;
+        for (int k = 0; k < n; ++k) sites += ctxs[k]->lat.Vh;
+        const int shape = bc.tuned ? bc.shape : sites >= 400000 ? shape_of_block(192) : 0;
         auto t0 = std::chrono::steady_clock::now();
-        if (inner == PLQ_F64) stt = launch_f64_18(a, bc.shape, bc.blocks_per_sm, s, bc, &lo);
-        else if (inner == PLQ_F32 && reals == 18) stt = launch_f32_18(a, bc.shape, bc.blocks_per_sm, s, bc, &lo);
-        else if (inner == PLQ_F32) stt = launch_f32_12(a, bc.shape, bc.blocks_per_sm, s, bc, &lo);
-        else stt = launch_f16_12(a, bc.shape, bc.blocks_per_sm, s, bc, &lo);
+        if (inner == PLQ_F64) stt = launch_f64_18(a, shape, bc.blocks_per_sm, s, bc, &lo);
+        else if (inner == PLQ_F32 && reals == 18) stt = launch_f32_18(a, shape, bc.blocks_per_sm, s, bc, &lo);
+        else if (inner == PLQ_F32) stt = launch_f32_12(a, shape, bc.blocks_per_sm, s, bc, &lo);
+        else stt = launch_f16_12(a, shape, bc.blocks_per_sm, s, bc, &lo);
         if (stt != PLQ_OK) break;
         int status_word = 0;
         e = cudaMemcpyAsync(res.data(), a.res, bytes_res, cudaMemcpyDeviceToHost, s);
@@ -209,12 +226,6 @@ extern "C" plq_status plq_cg_solve_batched(plq_ctx **ctxs, int n, void **x, cons
 }
 
 namespace {
-
-int shape_of_block(int block) {
-    for (int k = 0; k < kNumShapes; ++k)
-        if (kShapes[k].block == block) return k;
-    return -1;
-}
 
 // "GPU|batched|inner|links|n|lattice,lattice,..." (lattices in batch order)
 std::string batch_key(plq_ctx **ctxs, int n, int inner) {
@@ -297,6 +308,7 @@ extern "C" plq_status plq_autotune_batched(plq_ctx **ctxs, int n, void **x, cons
     // graph) and is timed on the second
     double best = 1e300;
     int best_shape = 0, best_bps = 0;
+    bc.tuned = 1;  // the solves below run in the shape set here
     plq_batch_info bestbi{};
     for (int sh = 0; sh < kNumShapes; ++sh) {
         int full = 0;

@@ -43,7 +43,7 @@ struct BatchSystem {
     void *xe, *xo;
     int inner_scaled;  // 1: scale the inner iteration (FP32 / FP16 inner precision)
     void *bhat, *s64, *to64;           // FP64 half fields (to64: odd)
-    void *rL, *pL, *qL, *mpL, *toL;    // inner half fields (toL: odd)
+    void *rL, *pL, *mpL, *toL;    // inner half fields (toL: odd)
     void *xL;                          // inner solution accumulator (FP32 or FP64)
 };
 
@@ -64,9 +64,8 @@ enum Mode {
     M_IT1,         // to = H_oe p
     M_IT2,         // mp = p - kappa^2 H_eo to, |mp|^2 -> alpha
     M_IT3,         // to = D_oe mp
-    M_IT4,         // q = mp - kappa^2 D_eo to
-    M_IT5,         // x += alpha p, r -= alpha q, |r|^2 -> beta
-    M_IT6,         // p = r + beta p
+    M_IT4,         // r -= alpha (mp - kappa^2 D_eo to), |r|^2 -> beta
+    M_IT5,         // x += alpha p, p = r + beta p (unless the cycle ends here)
     M_ACC,         // x_e += xL (FP64)
     M_FIN1,        // x_o = b_o + kappa H_oe x_e (H_oe x_e of the last check, kept in to)
     M_ZERO,        // zero source: x_o = 0
@@ -78,6 +77,7 @@ enum { BF_NAN = 1, BF_NOT_CONVERGED = 2 };
 struct SysRun {
     int mode, iter, nrel, first, flags, reduces;
     int toe;    // to64 holds H_oe x_e of the current x_e
+    int last;   // this iteration ends the cycle: no new direction
     double b2, s2, r2, rho, alpha, beta, last_rho, stop_r2, target2, sigma;
     double sc;  // power of two applied where the residual enters the inner precision
 };
@@ -135,14 +135,18 @@ __device__ __forceinline__ void st(void *f, int Vh, int i, const cx<RealOf<P>> v
     Spinor<P>::store(f, (size_t)Vh, (size_t)i, v);
 }
 
+// v with its sign bit flipped where `flip` is 0x80000000: an integer operation
+// (negating a double that is not the operand of an addition or product costs an
+// instruction of the FP64 pipe).
+__device__ __forceinline__ double sign_flip(double v, unsigned flip) {
+    return __hiloint2double(__double2hiint(v) ^ (int)flip, __double2loint(v));
+}
+
 // z * i^k for a run-time k (0..3)
-template <class T>
-__device__ __forceinline__ cx<T> mul_ipow_rt(cx<T> z, int k) {
-    const bool sw = k & 1, neg_re = k == 1 || k == 2, neg_im = k >= 2;
-    cx<T> w = {sw ? z.im : z.re, sw ? z.re : z.im};
-    if (neg_re) w.re = -w.re;
-    if (neg_im) w.im = -w.im;
-    return w;
+__device__ __forceinline__ cx<double> mul_ipow_rt(cx<double> z, int k) {
+    const bool sw = k & 1;
+    const unsigned re = (k == 1 || k == 2) ? 0x80000000u : 0u, im = k >= 2 ? 0x80000000u : 0u;
+    return {sign_flip(sw ? z.im : z.re, re), sign_flip(sw ? z.re : z.im, im)};
 }
 
 // Direction d = 2 mu + back of one output site with every direction-dependent
@@ -156,6 +160,7 @@ template <int P, int R>
 __device__ __forceinline__ void hop_dir_rt(const Lattice &L, const char *g, size_t gb, int par, bool dag,
                                            const void *in, const SiteGeom &geo, int i, int d,
                                            cx<RealOf<P>> acc[12]) {
+    static_assert(P == PLQ_F64, "the FP64 phases");
     using T = RealOf<P>;
     const int mu = d >> 1;
     const bool back = d & 1;
@@ -180,8 +185,8 @@ __device__ __forceinline__ void hop_dir_rt(const Lattice &L, const char *g, size
 #pragma unroll
             for (int y = x; y < 3; ++y) {
                 const cx<T> p = u[x][y], q = u[y][x];
-                u[x][y] = {q.re, -q.im};
-                u[y][x] = {p.re, -p.im};
+                u[x][y] = {q.re, sign_flip(q.im, 0x80000000u)};
+                u[y][x] = {p.re, sign_flip(p.im, 0x80000000u)};
             }
     }
     const bool p2 = mu == 0 || mu == 3;
@@ -251,7 +256,7 @@ template <class T>
 __device__ __forceinline__ T norm12(const cx<T> v[12]) {
     T s = 0;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) s += v[k].re * v[k].re + v[k].im * v[k].im;
+    for (int k = 0; k < 12; ++k) s = fma(v[k].re, v[k].re, fma(v[k].im, v[k].im, s));
     return s;
 }
 
@@ -384,34 +389,32 @@ __device__ double run_site(int mode, const BatchSystem &B, const SysRun &R, int 
         const T a = (T)(-kk);
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = {fma(a, acc[k].re, x[k].re), fma(a, acc[k].im, x[k].im)};
-        st<PL>(mode == M_IT2 ? B.mpL : B.qL, Vh, i, acc);
-        return mode == M_IT2 ? (double)norm12(acc) : 0.0;
+        if (mode == M_IT4) {  // the residual update, without storing Mhat^dagger Mhat p
+            const T al = -(T)R.alpha;
+            ld<PL>(B.rL, Vh, i, x);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) acc[k] = {fma(al, acc[k].re, x[k].re), fma(al, acc[k].im, x[k].im)};
+        }
+        st<PL>(mode == M_IT2 ? B.mpL : B.rL, Vh, i, acc);
+        return (double)norm12(acc);
     }
     case M_IT5: {
-        cx<T> p[12], q[12], r[12];
+        cx<T> p[12], r[12];
         cx<RealOf<PX>> x[12];
         ld<PL>(B.pL, Vh, i, p);
-        ld<PL>(B.qL, Vh, i, q);
-        ld<PL>(B.rL, Vh, i, r);
         ld<PX>(B.xL, Vh, i, x);
         const T al = (T)R.alpha;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
+        for (int k = 0; k < 12; ++k)
             x[k] = {fma((RealOf<PX>)al, (RealOf<PX>)p[k].re, x[k].re), fma((RealOf<PX>)al, (RealOf<PX>)p[k].im, x[k].im)};
-            r[k] = {fma(-al, q[k].re, r[k].re), fma(-al, q[k].im, r[k].im)};
-        }
         st<PX>(B.xL, Vh, i, x);
-        st<PL>(B.rL, Vh, i, r);
-        return (double)norm12(r);
-    }
-    case M_IT6: {
-        cx<T> p[12], r[12];
-        ld<PL>(B.pL, Vh, i, p);
-        ld<PL>(B.rL, Vh, i, r);
-        const T be = (T)R.beta;
+        if (!R.last) {
+            ld<PL>(B.rL, Vh, i, r);
+            const T be = (T)R.beta;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) p[k] = {fma(be, p[k].re, r[k].re), fma(be, p[k].im, r[k].im)};
-        st<PL>(B.pL, Vh, i, p);
+            for (int k = 0; k < 12; ++k) p[k] = {fma(be, p[k].re, r[k].re), fma(be, p[k].im, r[k].im)};
+            st<PL>(B.pL, Vh, i, p);
+        }
         return 0.0;
     }
     case M_ACC: {
@@ -441,7 +444,7 @@ __device__ double run_site(int mode, const BatchSystem &B, const SysRun &R, int 
 
 __device__ __forceinline__ bool reduces(int mode) {
     return mode == M_SETUP0 || mode == M_RES0 || mode == M_RES2 || mode == M_RES4 || mode == M_IT2 ||
-           mode == M_IT5;
+           mode == M_IT4;
 }
 
 // Deterministic state update after a phase, applied identically by every
@@ -489,23 +492,21 @@ __device__ inline void advance(SysRun &R, const BatchSystem &B, double v) {
         else R.mode = M_IT3;
         break;
     case M_IT3: R.mode = M_IT4; break;
-    case M_IT4: R.mode = M_IT5; break;
-    case M_IT5: {
+    case M_IT4: {
         const double rho_old = R.rho;
         R.beta = v / rho_old;
         R.rho = v;
         R.iter += 1;
         if (!isfinite(v)) { R.flags |= BF_NAN; R.mode = M_FIN1; break; }
-        if (v <= R.stop_r2 || R.iter >= B.maxit) {
+        R.last = v <= R.stop_r2 || R.iter >= B.maxit;
+        if (R.last) {
             R.last_rho = rho_old;  // |r|^2 of the iteration before the trigger
             if (v <= R.target2 * 1.0000001) R.sigma *= 0.25;
-            R.mode = M_ACC;
-        } else {
-            R.mode = M_IT6;
         }
+        R.mode = M_IT5;
         break;
     }
-    case M_IT6: R.mode = M_IT1; break;
+    case M_IT5: R.mode = R.last ? M_ACC : M_IT1; break;
     case M_ACC: R.nrel += 1; R.mode = M_RES1; break;
     case M_FIN1: R.mode = M_DONE; break;
     case M_ZERO: R.mode = M_DONE; break;
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) batched_cg_kernel(BatchArgs a) {
     for (int s = threadIdx.x; s < ns; s += blockDim.x) {
         SysRun R;
         R.mode = M_SETUP0;
-        R.iter = R.nrel = R.flags = R.reduces = R.toe = 0;
+        R.iter = R.nrel = R.flags = R.reduces = R.toe = R.last = 0;
         R.first = 1;
         R.b2 = R.s2 = R.r2 = R.rho = R.alpha = R.beta = R.last_rho = R.stop_r2 = R.target2 = 0.0;
         R.sigma = 0.5;
@@ -553,26 +554,41 @@ __global__ void __launch_bounds__(BLOCK, MINB) batched_cg_kernel(BatchArgs a) {
         __syncthreads();
         const long long total = prefix[ns];
         if (total == 0) break;  // every system retired
+        int ws = -1;        // the system whose sum wsum holds, the same in all lanes
+        double wsum = 0.0;
+        auto flush = [&]() {  // by whole warps
+            if (ws >= 0 && reduces(run[ws].mode)) {
+                double w = wsum;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+                if ((threadIdx.x & 31) == 0) atomicAdd(&bsum[ws], w);
+            }
+            wsum = 0.0;
+        };
         for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += stride) {
             int s = 0;
             while (g >= prefix[s + 1]) ++s;
             s = PLQ_GUARD(a.status, s, ns);
             const int i = PLQ_GUARD(a.status, (int)(g - prefix[s]), a.sys[s].lat.Vh);
             const double v = run_site<PL, RL>(run[s].mode, a.sys[s], run[s], i);
-            if (reduces(run[s].mode)) {
-                // warp-level sum when the whole warp works on one system
-                const unsigned m = __activemask();
-                const int s0 = __shfl_sync(m, s, __ffs(m) - 1);
-                if (__all_sync(m, s == s0) && m == 0xffffffffu) {
-                    double w = v;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(m, w, o);
-                    if ((threadIdx.x & 31) == 0) atomicAdd(&bsum[s], w);
-                } else {
-                    atomicAdd(&bsum[s], v);
+            // The sums of a warp that stays in one system are kept per thread and
+            // combined when it leaves the system: an addition per site instead of
+            // a shuffle tree and an atomic per 32 sites (16 cycles of the FP64 pipe
+            // for each instruction of them).
+            const unsigned m = __activemask();
+            const int s0 = __shfl_sync(m, s, __ffs(m) - 1);
+            if (__all_sync(m, s == s0) && m == 0xffffffffu) {
+                if (ws != s0) {
+                    flush();
+                    ws = s0;
                 }
+                if (reduces(run[s].mode)) wsum += v;
+            } else if (reduces(run[s].mode)) {
+                atomicAdd(&bsum[s], v);
             }
         }
+        __syncwarp();
+        flush();
         __syncthreads();
         for (int s = threadIdx.x; s < ns; s += blockDim.x)
             if (run[s].mode != M_DONE && reduces(run[s].mode) && bsum[s] != 0.0) atomicAdd(&acc_now[s], bsum[s]);
