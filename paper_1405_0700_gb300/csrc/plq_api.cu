@@ -124,6 +124,19 @@ HopArgs hop_args(const plq_ctx *ctx, int prec, int out_parity, void *out, const 
     return a;
 }
 
+// out_p = x_p + a H_{p,1-p} in_{1-p} with x = in, for both parities.
+HopArgs both_parities(const plq_ctx *ctx, int prec, void *oe, const void *ie, void *oo, const void *io) {
+    HopArgs a = hop_args(ctx, prec, 0, oe, io);
+    const HopArgs b = hop_args(ctx, prec, 1, oo, ie);
+    a.x = ie;
+    a.both = 1;
+    a.in2 = b.in;
+    a.out2 = b.out;
+    a.nbr2 = b.nbr;
+    a.x2 = io;
+    return a;
+}
+
 }  // namespace
 
 extern "C" {
@@ -520,14 +533,9 @@ plq_status plq_wilson_apply(plq_ctx *c, void *out, const void *in, double kappa,
     const char *ie = static_cast<const char *>(in), *io = ie + half;
     char *oe = static_cast<char *>(out), *oo = oe + half;
     // out_e = in_e - kappa H_eo in_o ; out_o = in_o - kappa H_oe in_e
-    HopArgs a = hop_args(c, prec, 0, oe, io);
-    a.x = ie;
+    HopArgs a = both_parities(c, prec, oe, ie, oo, io);
     a.a = -kappa;
-    PLQ_TRY(launch_hop(a, prec, c->gauge[prec].reals, EPI_XPAY, s));
-    HopArgs b = hop_args(c, prec, 1, oo, ie);
-    b.x = io;
-    b.a = -kappa;
-    return launch_hop(b, prec, c->gauge[prec].reals, EPI_XPAY, s);
+    return launch_hop(a, prec, c->gauge[prec].reals, EPI_XPAY, s);
 }
 
 plq_status plq_twisted_apply(plq_ctx *c, void *out, const void *in, double kappa, double mu, int prec,
@@ -542,16 +550,10 @@ plq_status plq_twisted_apply(plq_ctx *c, void *out, const void *in, double kappa
     const char *ie = static_cast<const char *>(in), *io = ie + half;
     char *oe = static_cast<char *>(out), *oo = oe + half;
     // out_p = (1 + 2 i kappa mu gamma5) in_p - kappa H_{p,1-p} in_{1-p}
-    HopArgs a = hop_args(c, prec, 0, oe, io);
-    a.x = ie;
+    HopArgs a = both_parities(c, prec, oe, ie, oo, io);
     a.a = -kappa;
     a.nu_x = 2.0 * kappa * mu;
-    PLQ_TRY(launch_hop(a, prec, c->gauge[prec].reals, EPI_XPAY, s));
-    HopArgs b = hop_args(c, prec, 1, oo, ie);
-    b.x = io;
-    b.a = -kappa;
-    b.nu_x = 2.0 * kappa * mu;
-    return launch_hop(b, prec, c->gauge[prec].reals, EPI_XPAY, s);
+    return launch_hop(a, prec, c->gauge[prec].reals, EPI_XPAY, s);
 }
 
 plq_status plq_schur_apply(plq_ctx *c, void *out, const void *in, void *tmp, double kappa, int dagger, int prec,

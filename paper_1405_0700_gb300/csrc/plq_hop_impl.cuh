@@ -933,12 +933,23 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
     // neighbour-table variants for the plain and xpay epilogues; the
     // row-streamed kernel for whole-lattice applications with those epilogues.
     if (a.smem_links == 5 || a.untuned) {
-        if (split_fits(a, epi) && (a.smem_links == 5 || split_default<P>(a))) return dispatch_split<P, R>(a, epi, s);
+        if (split_fits(a, epi) && (a.smem_links == 5 || split_default<P>(a, epi))) return dispatch_split<P, R>(a, epi, s);
         if (a.smem_links == 5) {  // a tuned split launch, where the split kernel has no form: the library's default
             HopArgs d = a;
             d.smem_links = d.block = 0;
             return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
         }
+    }
+    if (a.both) {  // the parities one after the other
+        HopArgs h = a;
+        h.both = 0;
+        PLQ_TRY((dispatch_hop<P, R>(h, epi, s, block)));
+        h.in = a.in2;
+        h.x = a.x2;
+        h.out = a.out2;
+        h.nbr = a.nbr2;
+        h.out_parity = 1 - a.out_parity;
+        return dispatch_hop<P, R>(h, epi, s, block);
     }
     if constexpr (P != PLQ_F64) {
         // Links staged in shared memory or read by every right-hand side's thread:

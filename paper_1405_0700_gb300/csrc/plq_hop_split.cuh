@@ -16,7 +16,8 @@
 // grid leave a nearly empty second wave.  Two applications (plq_schur_apply),
 // hop_kernel -> this: FP64 8^4 71 -> 25 us, 12^3x16 70 -> 56, 16^3x32 253 -> 226,
 // 24^3x32 745 -> 725, 24^3x48 1110 -> 1079 us; one application 32^3x64 1628 ->
-// 1619 us, 24^3x48 with 12 right-hand sides 6167 -> 6132 us.  Three blocks per SM
+// 1619 us, 24^3x48 with 12 right-hand sides 6167 -> 6132 us; both parities in one
+// launch (plq_wilson_apply) 16^3x32 236 -> 217 us.  Three blocks per SM
 // with a few spilled registers beat two without (16^3x32 230, 24^3x48 1102 us).
 //
 // FP32 and FP16 storage are bound by memory or issue beyond small lattices and
@@ -146,12 +147,24 @@ constexpr long long kSplitElements = 8192;
 // The reducing epilogues keep one right-hand side per thread: one in all.
 inline bool split_fits(const HopArgs &a, int epi) { return a.nrhs == 1 || epi <= EPI_XPAY; }
 
+// FP64 with a norm: 16^3x32 (65,536 sites) 142 us in hop_kernel, 130 here, but
+// 24^3x48 (331,776) 580 against 616 us, where blocks walk several tiles.
 template <int P>
-bool split_default(const HopArgs &a) {
-    return P == PLQ_F64 || (long long)a.lat.Vh * a.nrhs <= kSplitElements;
+bool split_default(const HopArgs &a, int epi) {
+    if (P == PLQ_F64) return epi < EPI_XPAY_NORM || a.lat.Vh <= 131072;
+    return (long long)a.lat.Vh * a.nrhs <= kSplitElements;
 }
-template <int P, int R, int EPI, bool DAG>
-__global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY_NORM ? 3 : 4) hop_split_kernel(const HopArgs a) {
+
+// Args: one launch, or the launches of both parities (blockIdx.y picks).
+struct HopPair {
+    HopArgs a[2];
+};
+template <int P, int R, int EPI, bool DAG, class Args>
+__global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY_NORM ? 3 : 4) hop_split_kernel(const Args args) {
+    const HopArgs &a = [&]() -> const HopArgs & {
+        if constexpr (sizeof(Args) == sizeof(HopPair)) return args.a[blockIdx.y];
+        else return args;
+    }();
     using T = RealOf<P>;
     using PL = Plane<T>;
     using V = typename PL::V;
@@ -268,15 +281,23 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
     if constexpr (NV > 0) grid_reduce(a.red, racc, 1);
 }
 
-template <int P, int R, int EPI, bool DAG>
+template <int P, int R, int EPI, bool DAG, bool BOTH = false>
 plq_status launch_split_t(const HopArgs &a, cudaStream_t s) {
-    auto kern = hop_split_kernel<P, R, EPI, DAG>;
     const int i_end = a.site_end < 0 ? a.lat.Vh : a.site_end;
     long long grid = ((long long)(i_end - a.site_begin) * a.nrhs + 31) / 32;
     if (grid <= 0) return PLQ_OK;
     // reducing launches: every block adds partial sums
     if (EPI >= EPI_XPAY_NORM && grid > kMaxReduceBlocks / 2) grid = kMaxReduceBlocks / 2;
-    kern<<<(unsigned)grid, kSplitThreads, 0, s>>>(a);
+    if constexpr (BOTH) {
+        HopPair p{{a, a}};
+        p.a[1].in = a.in2;
+        p.a[1].x = a.x2;
+        p.a[1].out = a.out2;
+        p.a[1].out_parity = 1 - a.out_parity;
+        hop_split_kernel<P, R, EPI, DAG, HopPair><<<dim3((unsigned)grid, 2), kSplitThreads, 0, s>>>(p);
+    } else {
+        hop_split_kernel<P, R, EPI, DAG, HopArgs><<<(unsigned)grid, kSplitThreads, 0, s>>>(a);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "hop_split_kernel launch");
     return PLQ_OK;
@@ -284,6 +305,7 @@ plq_status launch_split_t(const HopArgs &a, cudaStream_t s) {
 
 template <int P, int R>
 plq_status dispatch_split(const HopArgs &a, int epi, cudaStream_t s) {
+    if (a.both && epi == EPI_XPAY && !a.dagger) return launch_split_t<P, R, EPI_XPAY, false, true>(a, s);
     switch (epi) {
     case EPI_PLAIN: return a.dagger ? launch_split_t<P, R, EPI_PLAIN, true>(a, s) : launch_split_t<P, R, EPI_PLAIN, false>(a, s);
     case EPI_XPAY: return a.dagger ? launch_split_t<P, R, EPI_XPAY, true>(a, s) : launch_split_t<P, R, EPI_XPAY, false>(a, s);

@@ -251,6 +251,12 @@ struct HopArgs {
     // neighbour, with bit 31 set when the hop crosses the time boundary.  NULL:
     // neighbours are computed from the coordinates.
     const int *nbr = nullptr;
+    // both = 1: the other parity too, with these (plq_wilson_apply: two independent
+    // half-lattice applications, one launch where the kernel has that form)
+    int both = 0;
+    const void *in2 = nullptr, *x2 = nullptr;
+    void *out2 = nullptr;
+    const int *nbr2 = nullptr;
     int block = 0;  // threads per block; 0 = default
     int rhs_tile = 1;  // right-hand sides per thread (1, 2 or 4; must divide nrhs)
     // Site order: 0 = checkerboard order (t slowest).  zc > 0 walks the lattice
