@@ -506,7 +506,8 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
             if (RT > 1 && a.st != nullptr && a.st[rr].stop) continue;
             const long long idx = PLQ_GUARD(a.kstatus, (long long)i * n + rr, (long long)stride);
             hop_epilogue<P, EPI>(a, stride, idx, rr, acc[t], racc, t);
-            Spinor<P>::store(a.out, stride, (size_t)idx, acc[t]);
+            if constexpr (P == PLQ_F16 && (R == 18 || EPI == EPI_XPAY)) Spinor<P>::store_flat(a.out, stride, (size_t)idx, acc[t]);
+            else Spinor<P>::store(a.out, stride, (size_t)idx, acc[t]);
         }
     }
     if constexpr (NV > 0) grid_reduce(a.red, racc, blockDim.x);
@@ -519,12 +520,15 @@ __device__ __forceinline__ void hop_body(const HopArgs &a) {
 // for resident warps, i.e. more bytes in flight per SM.  The values are the
 // fastest of a sweep (64..112) on the 32^3x64 half-application: 80 for FP32
 // with 18-real links, 72 for the other FP32/FP16 formats, 96 for the
-// epilogue kernels of the solvers.  FP64 is bound by its arithmetic and
+// epilogue kernels of the solvers but 80 for the plain FP32 xpay with 12-real
+// links (plq_wilson_apply on 24^3x48 78.7 -> 74.2 us; with 18-real links 94.8 ->
+// 113 us, FP16 54.1 / 61.4 -> 60.3 / 69.1 us, and the reducing kernels lose too).  FP64 is bound by its arithmetic and
 // runs uncapped, as do the neighbour-table variants (~72 registers anyway)
 // and the RHS-tiled kernels, whose tiles live in registers.
 template <int P, int R, int EPI, bool TBL, int RT>
 constexpr int hop_reg_cap() {
     if (RT != 1 || TBL || P == PLQ_F64) return 0;
+    if (EPI == EPI_XPAY && P == PLQ_F32 && R == 12) return 80;
     if (EPI != EPI_PLAIN) return 96;
     return (P == PLQ_F32 && R == 18) ? 80 : 72;
 }
