@@ -48,6 +48,30 @@ __device__ __forceinline__ cx<R> mul_ipow(cx<R> z) {
     else return {z.im, -z.re};
 }
 
+// ---------------------------------------------------------------- launches
+// Kernels of a chain begin with chain_begin() and are launched by
+// launch_chained (programmatic dependent launch): the next kernel's blocks come
+// onto the SMs as soon as this one's have all started and leave room, and wait
+// there for its completion, instead of being launched after it.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // ---------------------------------------------------------------- loads
 // Read-only, L1-cacheable (neighbour spinors are reused by up to 8 sites).
 __device__ __forceinline__ float4 ld_nc(const float4 *p) { return __ldg(p); }

@@ -37,6 +37,18 @@ __device__ __forceinline__ void twist12(cx<T> v[12], T nu, T scale) {
     }
 }
 
+// Whether a one-RHS launch is chained (launch_chained): operator calls in FP32
+// and FP64.  One after the other, hop_kernel -> chained: FP32 18-real 32^3x64 121.3
+// -> 119.1 us, 24^3x48 37.3 -> 34.9 us, plq_schur_apply on 24^3x48 86.6 -> 83.0 and
+// on 16^4 16.6 -> 12.8-14.2 us, FP64 on 16^4 119.4 -> 114.1 us.  The iterations of
+// the solvers, captured in graphs, lost (mixed CG on 24^3x48 15.87 -> 16.12 ms), and
+// so did several right-hand sides (3: 76.3 -> 77.7 us) and FP16 storage
+// (plq_schur_apply on 24^3x48 56.3 -> 59.3 us); they run unchained.
+template <int P>
+__host__ __device__ __forceinline__ bool chained(const HopArgs &a) {
+    return P != PLQ_F16 && a.st == nullptr && a.nrhs == 1;
+}
+
 // Scalars of a launch in the arithmetic of the kernel.
 template <class T>
 __device__ __forceinline__ T hop_a(const HopArgs &a) {
@@ -535,11 +547,13 @@ constexpr int hop_reg_cap() {
 
 template <int P, int R, int EPI, bool DAG, bool TBL, int RT = 1>
 __global__ void __launch_bounds__(256) hop_kernel(const HopArgs a) {
+    if (chained<P>(a)) chain_begin();
     hop_body<P, R, EPI, DAG, TBL, RT>(a);
 }
 
 template <int P, int R, int EPI, bool DAG, bool TBL, int RT, int NREG>
 __global__ void __maxnreg__(NREG) hop_kernel_capped(const HopArgs a) {
+    if (chained<P>(a)) chain_begin();
     hop_body<P, R, EPI, DAG, TBL, RT>(a);
 }
 
@@ -901,8 +915,7 @@ plq_status launch_hop_t(const HopArgs &a, cudaStream_t s, int block) {
     const int grid = (int)(want < cap ? want : cap);
     if (grid <= 0) return PLQ_OK;
     const dim3 bdim(tiles, spb);
-    kern<<<grid, bdim, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(chained<P>(a), kern, dim3(grid), bdim, s, a);
     if (e != cudaSuccess) return cuda_error(e, "hop_kernel launch");
     return PLQ_OK;
 }

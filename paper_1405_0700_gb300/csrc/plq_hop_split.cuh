@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(kSplitThreads, P == PLQ_F64 || EPI >= EPI_XPAY
         if constexpr (sizeof(Args) == sizeof(HopPair)) return args.a[blockIdx.y];
         else return args;
     }();
+    if (chained<P>(a)) chain_begin();
     using T = RealOf<P>;
     using PL = Plane<T>;
     using V = typename PL::V;
@@ -288,17 +289,18 @@ plq_status launch_split_t(const HopArgs &a, cudaStream_t s) {
     if (grid <= 0) return PLQ_OK;
     // reducing launches: every block adds partial sums
     if (EPI >= EPI_XPAY_NORM && grid > kMaxReduceBlocks / 2) grid = kMaxReduceBlocks / 2;
+    cudaError_t e;
     if constexpr (BOTH) {
         HopPair p{{a, a}};
         p.a[1].in = a.in2;
         p.a[1].x = a.x2;
         p.a[1].out = a.out2;
         p.a[1].out_parity = 1 - a.out_parity;
-        hop_split_kernel<P, R, EPI, DAG, HopPair><<<dim3((unsigned)grid, 2), kSplitThreads, 0, s>>>(p);
+        e = launch_chained(chained<P>(a), hop_split_kernel<P, R, EPI, DAG, HopPair>, dim3((unsigned)grid, 2), dim3(kSplitThreads), s, p);
     } else {
-        hop_split_kernel<P, R, EPI, DAG, HopArgs><<<(unsigned)grid, kSplitThreads, 0, s>>>(a);
+        e = launch_chained(chained<P>(a), hop_split_kernel<P, R, EPI, DAG, HopArgs>, dim3((unsigned)grid),
+                           dim3(kSplitThreads), s, a);
     }
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "hop_split_kernel launch");
     return PLQ_OK;
 }
