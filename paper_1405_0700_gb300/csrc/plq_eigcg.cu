@@ -14,12 +14,14 @@
 // x0 = U H^{-1} U^H rhs ("init-CG").
 //
 // GPU mapping: the CG iterations are the fused kernels of the other solvers,
-// captured in CUDA graphs; each iteration also copies r_{j+1} into its slot
-// of V, and the device records alpha_j, beta_j, |r_{j+1}|^2, so the host
-// builds T without stopping the GPU.  Restarts and Ritz extraction are a
-// small dense eigenproblem on the host (Jacobi, at most m = 64) and one
-// linear-combination kernel over V on the device; Gram-Schmidt and the
-// projections onto U are multi-vector dot / axpy kernels.
+// launched in batches that fill the search space; each iteration also copies
+// r_{j+1} into its slot of V, and the device records alpha_j, beta_j,
+// |r_{j+1}|^2, from which the host builds T.  Restarts and Ritz extraction are
+// a small dense eigenproblem on the host (Jacobi, at most m = 64, some 10 ms)
+// and one linear-combination kernel over V on the device.  CG itself does not
+// depend on them: the next batch is launched first and runs meanwhile
+// (16^3x32, nev = 10, m = 60, three sources: 251 -> 221 ms).  Gram-Schmidt and
+// the projections onto U are multi-vector dot / axpy kernels.
 //
 // Precision.  The CG iterations, H = U^H A U, the Galerkin start and every
 // residual are FP64.  The search space V (Lanczos vectors, restarts, Ritz
@@ -581,12 +583,71 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
         std::vector<SolverState> cur(1);
         bool converged = rho0 <= init.stop_r2;
         int ritz_k = 0;  // complete vectors in V at the end
+        // Rayleigh-Ritz on the full search space: E->V -> the first k2 slots of
+        // E->V2, whose later slots take the residuals that follow; the two swap
+        bool restart = false;
+        auto restart_space = [&]() -> plq_status {
+            std::vector<double> Tm((size_t)m * m);
+            for (int i2 = 0; i2 < m; ++i2)
+                for (int j2 = 0; j2 < m; ++j2) Tm[(size_t)i2 * m + j2] = T[(size_t)i2 * (m + 1) + j2];
+            std::vector<double> wv, Y, w2, Y2;
+            jacobi_eigh(m, Tm, wv, Y);
+            std::vector<double> Tm1((size_t)(m - 1) * (m - 1));
+            for (int i2 = 0; i2 < m - 1; ++i2)
+                for (int j2 = 0; j2 < m - 1; ++j2) Tm1[(size_t)i2 * (m - 1) + j2] = Tm[(size_t)i2 * m + j2];
+            jacobi_eigh(m - 1, Tm1, w2, Y2);
+            std::vector<double> Qm((size_t)m * k2, 0.0);
+            for (int i2 = 0; i2 < m; ++i2)
+                for (int l = 0; l < nev; ++l) {
+                    Qm[(size_t)i2 * k2 + l] = Y[(size_t)i2 * m + l];
+                    Qm[(size_t)i2 * k2 + nev + l] = i2 < m - 1 ? Y2[(size_t)i2 * (m - 1) + l] : 0.0;
+                }
+            orthonormalize_columns(m, k2, Qm);
+            std::vector<double> Hq((size_t)k2 * k2, 0.0), TQ((size_t)m * k2, 0.0);
+            for (int i2 = 0; i2 < m; ++i2)
+                for (int l = 0; l < k2; ++l) {
+                    double sacc = 0;
+                    for (int j2 = 0; j2 < m; ++j2) sacc += Tm[(size_t)i2 * m + j2] * Qm[(size_t)j2 * k2 + l];
+                    TQ[(size_t)i2 * k2 + l] = sacc;
+                }
+            for (int a2 = 0; a2 < k2; ++a2)
+                for (int b2 = 0; b2 < k2; ++b2) {
+                    double sacc = 0;
+                    for (int i2 = 0; i2 < m; ++i2) sacc += Qm[(size_t)i2 * k2 + a2] * TQ[(size_t)i2 * k2 + b2];
+                    Hq[(size_t)a2 * k2 + b2] = sacc;
+                }
+            std::vector<double> Mv, Z;
+            jacobi_eigh(k2, Hq, Mv, Z);
+            std::vector<double> QZ((size_t)m * k2, 0.0), C((size_t)m * k2);
+            for (int i2 = 0; i2 < m; ++i2)
+                for (int l = 0; l < k2; ++l) {
+                    double sacc = 0;
+                    for (int j2 = 0; j2 < k2; ++j2) sacc += Qm[(size_t)i2 * k2 + j2] * Z[(size_t)j2 * k2 + l];
+                    QZ[(size_t)i2 * k2 + l] = sacc;
+                    C[(size_t)i2 * k2 + l] = sacc / nrm[i2];  // raw slots -> normalised V
+                }
+            PLQ_TRY(rcomb(G, E->V, m, C, k2, E->V2));
+            PLQ_CUDA(cudaMemcpyAsync(E->V2 + (size_t)k2 * E->slot, E->V + (size_t)m * E->slot,
+                                     G.N * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+            std::swap(E->V, E->V2);
+            const double tlast = -std::sqrt(beta_prev) / alpha_prev;
+            std::fill(T.begin(), T.end(), 0.0);
+            for (int l = 0; l < k2; ++l) {
+                T[(size_t)l * (m + 1) + l] = Mv[l];
+                const double cpl = tlast * QZ[(size_t)(m - 1) * k2 + l];
+                T[(size_t)k2 * (m + 1) + l] = cpl;
+                T[(size_t)l * (m + 1) + k2] = cpl;
+                nrm[l] = 1.0;
+            }
+            nrm[k2] = nrm[m];
+            return PLQ_OK;
+        };
         while (!converged && iters < maxit && st == PLQ_OK) {
             init.iter = iters;
             std::vector<SolverState> sv(1, init);
             if ((st = put_states(G.S, sv)) != PLQ_OK) break;
             const int L = eig ? (m - vs + 1) : 16;
-            float2 *Vb = E->V;
+            float2 *Vb = restart ? E->V2 : E->V;
             auto body = [&](int i) -> plq_status {
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, p, EPI_PLAIN, 0, nullptr, 0.0, FIN_NONE, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, mp, to, EPI_XPAY_NORM, 0, p, -kk, FIN_CG_ALPHA, nullptr, true));
@@ -599,24 +660,10 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 }
                 return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s);
             };
-            // one graph of exactly L iterations (the ones that fill V)
-            cudaGraph_t graph = nullptr;
-            cudaGraphExec_t exec = nullptr;
-            PLQ_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
             for (int i = 0; i < L && st == PLQ_OK; ++i) st = body(i);
-            cudaError_t ce = cudaStreamEndCapture(s, &graph);
-            if (st != PLQ_OK) {
-                if (graph) cudaGraphDestroy(graph);
-                break;
-            }
-            if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
-            if (graph) cudaGraphDestroy(graph);
-            if (ce == cudaSuccess) ce = cudaGraphLaunch(exec, s);
-            if (exec) cudaGraphExecDestroy(exec);
-            if (ce != cudaSuccess) {
-                st = cuda_error(ce, "EigCG iteration graph");
-                break;
-            }
+            if (st == PLQ_OK && restart) st = restart_space();
+            restart = false;
+            if (st != PLQ_OK) break;
             if ((st = get_states(G.S, cur)) != PLQ_OK) break;
             const int done = cur[0].iter - iters;
             if (cur[0].flags & FLAG_NAN) {
@@ -645,60 +692,8 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 }
                 ritz_k = vs - 1 + done;  // complete vectors
                 if (!converged && ritz_k == m && iters + done < maxit) {
-                    // restart with 2 nev Ritz vectors
-                    std::vector<double> Tm((size_t)m * m);
-                    for (int i2 = 0; i2 < m; ++i2)
-                        for (int j2 = 0; j2 < m; ++j2) Tm[(size_t)i2 * m + j2] = T[(size_t)i2 * (m + 1) + j2];
-                    std::vector<double> wv, Y, w2, Y2;
-                    jacobi_eigh(m, Tm, wv, Y);
-                    std::vector<double> Tm1((size_t)(m - 1) * (m - 1));
-                    for (int i2 = 0; i2 < m - 1; ++i2)
-                        for (int j2 = 0; j2 < m - 1; ++j2) Tm1[(size_t)i2 * (m - 1) + j2] = Tm[(size_t)i2 * m + j2];
-                    jacobi_eigh(m - 1, Tm1, w2, Y2);
-                    std::vector<double> Qm((size_t)m * k2, 0.0);
-                    for (int i2 = 0; i2 < m; ++i2)
-                        for (int l = 0; l < nev; ++l) {
-                            Qm[(size_t)i2 * k2 + l] = Y[(size_t)i2 * m + l];
-                            Qm[(size_t)i2 * k2 + nev + l] = i2 < m - 1 ? Y2[(size_t)i2 * (m - 1) + l] : 0.0;
-                        }
-                    orthonormalize_columns(m, k2, Qm);
-                    std::vector<double> Hq((size_t)k2 * k2, 0.0), TQ((size_t)m * k2, 0.0);
-                    for (int i2 = 0; i2 < m; ++i2)
-                        for (int l = 0; l < k2; ++l) {
-                            double sacc = 0;
-                            for (int j2 = 0; j2 < m; ++j2) sacc += Tm[(size_t)i2 * m + j2] * Qm[(size_t)j2 * k2 + l];
-                            TQ[(size_t)i2 * k2 + l] = sacc;
-                        }
-                    for (int a2 = 0; a2 < k2; ++a2)
-                        for (int b2 = 0; b2 < k2; ++b2) {
-                            double sacc = 0;
-                            for (int i2 = 0; i2 < m; ++i2) sacc += Qm[(size_t)i2 * k2 + a2] * TQ[(size_t)i2 * k2 + b2];
-                            Hq[(size_t)a2 * k2 + b2] = sacc;
-                        }
-                    std::vector<double> Mv, Z;
-                    jacobi_eigh(k2, Hq, Mv, Z);
-                    std::vector<double> QZ((size_t)m * k2, 0.0), C((size_t)m * k2);
-                    for (int i2 = 0; i2 < m; ++i2)
-                        for (int l = 0; l < k2; ++l) {
-                            double sacc = 0;
-                            for (int j2 = 0; j2 < k2; ++j2) sacc += Qm[(size_t)i2 * k2 + j2] * Z[(size_t)j2 * k2 + l];
-                            QZ[(size_t)i2 * k2 + l] = sacc;
-                            C[(size_t)i2 * k2 + l] = sacc / nrm[i2];  // raw slots -> normalised V
-                        }
-                    if ((st = rcomb(G, E->V, m, C, k2, E->V2)) != PLQ_OK) break;
-                    PLQ_CUDA(cudaMemcpyAsync(E->V2 + (size_t)k2 * E->slot, E->V + (size_t)m * E->slot,
-                                             G.N * sizeof(float2), cudaMemcpyDeviceToDevice, s));
-                    std::swap(E->V, E->V2);
-                    const double tlast = -std::sqrt(beta_prev) / alpha_prev;
-                    std::fill(T.begin(), T.end(), 0.0);
-                    for (int l = 0; l < k2; ++l) {
-                        T[(size_t)l * (m + 1) + l] = Mv[l];
-                        const double cpl = tlast * QZ[(size_t)(m - 1) * k2 + l];
-                        T[(size_t)k2 * (m + 1) + l] = cpl;
-                        T[(size_t)l * (m + 1) + k2] = cpl;
-                        nrm[l] = 1.0;
-                    }
-                    nrm[k2] = nrm[m];
+                    // restart with 2 nev Ritz vectors, behind the launches of the next batch
+                    restart = true;
                     vs = k2 + 1;
                 } else {
                     vs = ritz_k + 1;

@@ -5,6 +5,7 @@ import pytest
 import synthetic as S
 from gpuhelp import TOL, gpu_hopping_full, rel
 from oracle import c_oracle as C
+from oracle import wilson as W
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -139,3 +140,45 @@ def test_calls_follow_the_current_stream():
             assert plq._stream(None) == side.cuda_stream == torch.cuda.current_stream().cuda_stream
         assert plq._stream(None) == torch.cuda.current_stream().cuda_stream
     assert plq._stream(side) == side.cuda_stream and plq._stream(5) == 5
+
+
+# the inner products, search-space slots and restarts of EigCG: one vector, counts around the
+# 16 of a launch, restarts every two iterations, fields of less than a block and of several
+# elements a thread.  Eigenvalues of H = U^H A U lie within the spectrum of A up to
+# |U^H U - 1| <= k 4 2^-24 < 1e-5 (k <= 40 vectors orthonormalised in FP32); a sum that misses
+# a term, a slot overwritten or a restart from the wrong slots leaves vectors that are not
+# orthonormal or an H that is not theirs.
+@pytest.mark.parametrize("dims,unit,nev,m,solves", [((4, 2, 2, 2), False, 1, 4, 18), ((4, 4, 2, 6), False, 6, 14, 6),
+                                                    ((16, 8, 8, 16), True, 8, 20, 3)])
+def test_eigcg_basis(dims, unit, nev, m, solves):
+    kappa = 0.115
+    U = S.gauge_field(dims, 0.3, 23)
+    if unit:  # free field: A is diagonal in momentum space, 1 - kappa^2 H(p)^2 with H(p) = a +- i |b|
+        U = np.zeros_like(U) + np.eye(3)
+        # (antiperiodic in time: half-integer momenta)
+        p = np.meshgrid(*[2 * np.pi * (np.arange(n) + 0.5 * (i == 0)) / n for i, n in enumerate(dims)], indexing="ij")
+        h = 2 * sum(np.cos(q) for q in p) + 2j * np.sqrt(sum(np.sin(q) ** 2 for q in p))
+        lam = np.abs(1 - kappa**2 * h**2) ** 2
+    else:
+        even = W.parity(S.lattice_shape(dims)) == 0
+        n = int(even.sum()) * 12
+        A = np.empty((n, n), dtype=np.complex128)
+        for k in range(n):
+            v = np.zeros(S.lattice_shape(dims) + (4, 3), dtype=np.complex128)
+            v[even] = np.eye(n)[k].reshape(-1, 4, 3)
+            A[:, k] = W.schur_dag(U, W.schur(U, v, kappa), kappa)[even].ravel()
+        lam = np.linalg.eigvalsh(A)
+    with Context(dims) as ctx:
+        ctx.gauge_upload(U, 18, F64)
+        eig = plq.EigCG(ctx, nev=nev, m=m, max_vectors=nev * solves)
+        x = ctx.empty_full(F64)
+        for k in range(solves + 1):
+            info = eig.solve(x, ctx.to_device(S.gaussian_spinor(dims, 700 + k), F64), kappa, tol=1e-11)
+            # |r_x| <= |Mhat^-dag| |r_normal|, |rhs| <= |Mhat| |bhat| and |bhat| <= (1 + 8 kappa) |b|
+            assert info.true_rel_residual <= 1.01e-11 * np.sqrt(lam.max() / lam.min()) * (1 + 8 * kappa)
+        held, H = eig.vectors, eig.projected_matrix()
+        eig.close()
+    assert held == nev * solves
+    theta = np.linalg.eigvalsh(H)
+    assert np.allclose(H, H.conj().T, atol=1e-14)
+    assert theta[0] >= lam.min() * (1 - 1e-5) and theta[-1] <= lam.max() * (1 + 1e-5), (theta[0], lam.min())
