@@ -161,12 +161,11 @@ bool chol_solve(int n, const std::vector<std::complex<double>> &Hm, int ld, std:
 }
 
 // ---------------------------------------------------------------- device kernels
-int grid_of(long long work, bool reduce) {
+int grid_of(long long work, int per_sm = 8) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    long long want = (work + 255) / 256, cap = (long long)sms * 8;
-    if (reduce && cap > kMaxReduceBlocks) cap = kMaxReduceBlocks;
+    long long want = (work + 255) / 256, cap = (long long)sms * per_sm;
     if (want < 1) want = 1;
     return (int)(want < cap ? want : cap);
 }
@@ -229,17 +228,46 @@ __global__ void zlincomb32_kernel(long long N, const float2 *in, size_t stride, 
     }
 }
 
-// d_i = <u_i, w> for i < cnt (<= kDotChunk), FP32 slots; per-thread FP32 partial
-// sums (a handful of elements each), FP64 across threads and blocks
-__global__ void multidot32_kernel(long long N, const float2 *U, size_t stride, int cnt, const float2 *w, Reduce red) {
-    RedAcc<2 * kDotChunk> acc;
-    red_init(acc);
+// What one element adds to (re, im) of <a, b>.  FP64: two fused multiply-adds a
+// component.  FP32: the sums stay exact to ~2^-47 (SumFF) and take the rounding
+// error of one of the two products along.
+__device__ __forceinline__ void dot_add(double &re, double &im, double2 a, double2 b) {
+    re = fma(a.x, b.x, fma(a.y, b.y, re));
+    im = fma(a.x, b.y, fma(-a.y, b.x, im));
+}
+__device__ __forceinline__ void dot_add(SumFF &re, SumFF &im, float2 a, float2 b) {
+    const float m = __fmul_rn(a.y, b.y), k = __fmul_rn(a.y, b.x);
+    re.add(fmaf(a.x, b.x, m), fmaf(a.y, b.y, -m));
+    im.add(fmaf(a.x, b.y, -k), -fmaf(a.y, b.x, -k));
+}
+
+// d_i = <u_i, w> for i < cnt <= C vectors in slots `stride` apart.  128 bytes of
+// an element's vectors are in flight together, so two blocks of 256 threads per
+// SM cover the latency, and few threads keep the reduction of 2 C values cheap.  FP64
+// slots are bound by the FP64 pipe (four instructions per element and vector,
+// 5.4 us per vector of a 16^3x32 half field), FP32 slots by L2 once their sums
+// leave that pipe; the accumulators are registers only because the loop over the
+// vectors is unrolled (a loop to cnt keeps them in local memory).  EigCG on
+// 16^3x32 (three sources, nev = 10, m = 60): 221 -> 209 ms against one kernel
+// with FP64 sums for both types and 2048 threads per SM.
+template <int C, class E, class V>
+__global__ void __launch_bounds__(256, 2)
+multidot_kernel(long long N, const E *U, size_t stride, int cnt, const E *w, Reduce red) {
+    constexpr int kFlight = C < 128 / (int)sizeof(E) ? C : 128 / (int)sizeof(E);
+    RedAcc<2 * C, 1, V> acc;
+#pragma unroll
+    for (int i = 0; i < 2 * C; ++i) acc.v[i][0] = V{};
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N; e += (long long)gridDim.x * blockDim.x) {
-        const float2 b = w[e];
-        for (int i = 0; i < cnt; ++i) {
-            const float2 a = __ldg(U + i * stride + e);
-            acc.v[2 * i][0] += a.x * b.x + a.y * b.y;
-            acc.v[2 * i + 1][0] += a.x * b.y - a.y * b.x;
+        const E b = w[e];
+#pragma unroll
+        for (int g = 0; g < C; g += kFlight) {
+            E a[kFlight];
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (g + i < cnt) a[i] = __ldg(U + (g + i) * stride + e);
+#pragma unroll
+            for (int i = 0; i < kFlight; ++i)
+                if (g + i < cnt) dot_add(acc.v[2 * (g + i)][0], acc.v[2 * (g + i) + 1][0], a[i], b);
         }
     }
     grid_reduce(red, acc, 1);
@@ -269,40 +297,36 @@ __global__ void zlincomb_kernel(long long N, const double2 *in, size_t stride, i
     }
 }
 
-// d_i = <u_i, w> for i < cnt (<= kDotChunk)
-__global__ void multidot_kernel(long long N, const double2 *U, size_t stride, int cnt, const double2 *w, Reduce red) {
-    RedAcc<2 * kDotChunk> acc;
-    red_init(acc);
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N; e += (long long)gridDim.x * blockDim.x) {
-        const double2 b = w[e];
-        for (int i = 0; i < cnt; ++i) {
-            const double2 a = __ldg(U + i * stride + e);
-            acc.v[2 * i][0] += a.x * b.x + a.y * b.y;
-            acc.v[2 * i + 1][0] += a.x * b.y - a.y * b.x;
-        }
-    }
-    grid_reduce(red, acc, 1);
-}
-
 struct Eig {
     plq_eigcg *E;
     Solve S;
     long long N;  // complex elements of a half field
 };
 
-plq_status dots(Eig &G, const double2 *Ubase, int cnt, const double2 *w, std::vector<std::complex<double>> &d) {
+// d_i = <u_i, w> for i < cnt
+template <class E, class V>
+plq_status dots(Eig &G, const E *Ubase, int cnt, const E *w, std::vector<std::complex<double>> &d) {
     d.assign(cnt, {0, 0});
+    const int grid = grid_of(G.N, 2);
     for (int c0 = 0; c0 < cnt; c0 += kDotChunk) {
         const int c = std::min(kDotChunk, cnt - c0);
+        const E *u = Ubase + c0 * G.E->slot;
         Reduce r = reduce_of(G.S.c, FIN_NONE);
         r.st = nullptr;
-        multidot_kernel<<<grid_of(G.N, true), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, c, w, r);
+        if (c == 1) multidot_kernel<1, E, V><<<grid, 256, 0, G.S.s>>>(G.N, u, G.E->slot, c, w, r);
+        else multidot_kernel<kDotChunk, E, V><<<grid, 256, 0, G.S.s>>>(G.N, u, G.E->slot, c, w, r);
         PLQ_CUDA(cudaGetLastError());
         double buf[2 * kDotChunk];
         PLQ_TRY(read_sums(G.S, buf, 2 * c));
         for (int i = 0; i < c; ++i) d[c0 + i] = {buf[2 * i], buf[2 * i + 1]};
     }
     return PLQ_OK;
+}
+plq_status dots(Eig &G, const double2 *Ubase, int cnt, const double2 *w, std::vector<std::complex<double>> &d) {
+    return dots<double2, double>(G, Ubase, cnt, w, d);
+}
+plq_status dots32(Eig &G, const float2 *Ubase, int cnt, const float2 *w, std::vector<std::complex<double>> &d) {
+    return dots<float2, SumFF>(G, Ubase, cnt, w, d);
 }
 
 // out = base + sum_i c_i U_i, in chunks
@@ -317,25 +341,10 @@ plq_status zcomb(Eig &G, const double2 *Ubase, const std::vector<std::complex<do
     for (int c0 = 0; c0 < cnt; c0 += kDotChunk) {
         const int k = std::min(kDotChunk, cnt - c0);
         PLQ_CUDA(cudaMemcpyAsync(cdev, c.data() + c0, k * sizeof(double2), cudaMemcpyHostToDevice, G.S.s));
-        zlincomb_kernel<<<grid_of(G.N, false), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, k, cdev,
+        zlincomb_kernel<<<grid_of(G.N), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, k, cdev,
                                                                 c0 == 0 ? base : out, out);
         PLQ_CUDA(cudaGetLastError());
         PLQ_CUDA(cudaStreamSynchronize(G.S.s));  // cdev is reused by the next chunk
-    }
-    return PLQ_OK;
-}
-
-plq_status dots32(Eig &G, const float2 *Ubase, int cnt, const float2 *w, std::vector<std::complex<double>> &d) {
-    d.assign(cnt, {0, 0});
-    for (int c0 = 0; c0 < cnt; c0 += kDotChunk) {
-        const int c = std::min(kDotChunk, cnt - c0);
-        Reduce r = reduce_of(G.S.c, FIN_NONE);
-        r.st = nullptr;
-        multidot32_kernel<<<grid_of(G.N, true), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, c, w, r);
-        PLQ_CUDA(cudaGetLastError());
-        double buf[2 * kDotChunk];
-        PLQ_TRY(read_sums(G.S, buf, 2 * c));
-        for (int i = 0; i < c; ++i) d[c0 + i] = {buf[2 * i], buf[2 * i + 1]};
     }
     return PLQ_OK;
 }
@@ -347,7 +356,7 @@ plq_status zcomb32(Eig &G, const float2 *Ubase, const std::vector<std::complex<d
     for (int c0 = 0; c0 < cnt; c0 += kDotChunk) {
         const int k = std::min(kDotChunk, cnt - c0);
         PLQ_CUDA(cudaMemcpyAsync(cdev, c.data() + c0, k * sizeof(double2), cudaMemcpyHostToDevice, G.S.s));
-        zlincomb32_kernel<<<grid_of(G.N, false), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, k, cdev,
+        zlincomb32_kernel<<<grid_of(G.N), 256, 0, G.S.s>>>(G.N, Ubase + c0 * G.E->slot, G.E->slot, k, cdev,
                                                                   w, w);
         PLQ_CUDA(cudaGetLastError());
         PLQ_CUDA(cudaStreamSynchronize(G.S.s));  // cdev is reused by the next chunk
@@ -360,7 +369,7 @@ plq_status rcomb(Eig &G, const float2 *in, int m, const std::vector<double> &C, 
     std::vector<float> Cf(C.begin(), C.begin() + (size_t)m * k);
     float *cdev = reinterpret_cast<float *>(G.E->coef);
     PLQ_CUDA(cudaMemcpyAsync(cdev, Cf.data(), sizeof(float) * m * k, cudaMemcpyHostToDevice, G.S.s));
-    lincomb32_kernel<<<grid_of(G.N, false), 256, 0, G.S.s>>>(G.N, in, G.E->slot, m, cdev, k, out, G.E->slot);
+    lincomb32_kernel<<<grid_of(G.N), 256, 0, G.S.s>>>(G.N, in, G.E->slot, m, cdev, k, out, G.E->slot);
     PLQ_CUDA(cudaGetLastError());
     PLQ_CUDA(cudaStreamSynchronize(G.S.s));
     return PLQ_OK;
@@ -394,9 +403,9 @@ plq_status add_to_basis(Eig &G, const float2 *src, int cnt, void *tmp_o, void *t
         PLQ_TRY(dots32(G, w32, 1, w32, nn));
         const double n2 = std::real(nn[0]);
         if (!(n2 > 1e-20)) continue;  // linearly dependent: skip
-        scale32_kernel<<<grid_of(G.N, false), 256, 0, G.S.s>>>(G.N, w32, (float)(1.0 / std::sqrt(n2)));
+        scale32_kernel<<<grid_of(G.N), 256, 0, G.S.s>>>(G.N, w32, (float)(1.0 / std::sqrt(n2)));
         PLQ_CUDA(cudaGetLastError());
-        to64_kernel<<<grid_of(G.N, false), 256, 0, G.S.s>>>(G.N, w, w32);
+        to64_kernel<<<grid_of(G.N), 256, 0, G.S.s>>>(G.N, w, w32);
         PLQ_CUDA(cudaGetLastError());
         PLQ_TRY(apply_A(G, Aw, w, tmp_o, tmp_e));
         std::vector<std::complex<double>> col;
@@ -567,7 +576,7 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
         std::vector<double> T((size_t)(m + 1) * (m + 1), 0.0), nrm(m + 1, 1.0);
         int vs = 1;  // V slot 0 holds r_0 (raw)
         if (eig) {
-            to32_kernel<<<grid_of(G.N, false), 256, 0, s>>>(G.N, E->V, static_cast<const double2 *>(r), vscale);
+            to32_kernel<<<grid_of(G.N), 256, 0, s>>>(G.N, E->V, static_cast<const double2 *>(r), vscale);
             PLQ_CUDA(cudaGetLastError());
             nrm[0] = vscale * std::sqrt(rho0);
         }
@@ -654,8 +663,8 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, mp, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, r, to, EPI_XPAY_RUPD, 1, mp, -kk, FIN_CG_BETA, r, true));
                 if (eig) {  // raw r_{j+1} into its (FP32) slot of the search space
-                    to32_kernel<<<grid_of(G.N, false), 256, 0, s>>>(G.N, Vb + (size_t)(vs + i) * E->slot,
-                                                                    static_cast<const double2 *>(r), vscale);
+                    to32_kernel<<<grid_of(G.N), 256, 0, s>>>(G.N, Vb + (size_t)(vs + i) * E->slot,
+                                                             static_cast<const double2 *>(r), vscale);
                     PLQ_CUDA(cudaGetLastError());
                 }
                 return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s);

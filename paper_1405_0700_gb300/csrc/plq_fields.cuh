@@ -444,11 +444,32 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *state, const 
 // the working precision (one site's 12 components) are added in FP64, and the
 // combination over threads, warps and blocks below runs in a fixed order, so
 // the sums are reproducible bit for bit for a given launch configuration.
-template <int NV, int RT = 1>
+template <int NV, int RT = 1, class V = double>
 struct RedAcc {
-    double v[NV][RT];
+    V v[NV][RT];
     __device__ __forceinline__ void add(int k, int t, double x) { v[k][t] += x; }
 };
+
+// A sum kept as an FP32 value and the FP32 sum of its rounding errors (Knuth's
+// two-sum): 2^-47 relative, in six FP32 instructions and none of the FP64 pipe.
+struct SumFF {
+    float s, c;
+    __device__ __forceinline__ void add(float x, float err) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)) + err;
+        s = t;
+    }
+};
+__device__ __forceinline__ SumFF operator+(SumFF a, const SumFF &b) {
+    a.add(b.s, b.c);
+    return a;
+}
+__device__ __forceinline__ double sum_value(const SumFF &a) { return isfinite(a.c) ? (double)a.s + (double)a.c : (double)a.s; }
+__device__ __forceinline__ double sum_value(double a) { return a; }
+__device__ __forceinline__ SumFF shfl_xor(const SumFF &a, int h) {
+    return {__shfl_xor_sync(0xffffffffu, a.s, h), __shfl_xor_sync(0xffffffffu, a.c, h)};
+}
+__device__ __forceinline__ double shfl_xor(double a, int h) { return __shfl_xor_sync(0xffffffffu, a, h); }
 
 // Linear thread index and thread count of a (possibly 2-D) block.
 __device__ __forceinline__ int ltid() { return threadIdx.y * blockDim.x + threadIdx.x; }
@@ -505,13 +526,13 @@ __device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const 
 // use recursive halving in each warp, 31 additions instead of 160.
 constexpr int kRedThreads = 256;
 
-template <int NV, int RT>
-__device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols, double *wv, double *slot) {
+template <int NV, int RT, class V = double>
+__device__ __forceinline__ void block_sums(const V (&w)[NV * RT], int ncols, double *wv, double *slot) {
     constexpr int W = NV * RT;
     const int tid = ltid(), lane = tid & 31, warp = tid >> 5, nthr = lsize(), nw = (nthr + 31) >> 5;
     const int n = ncols * RT;
     if constexpr (W == 32) {  // one column, whole warps
-        double x[W];
+        V x[W];
 #pragma unroll
         for (int k = 0; k < W; ++k) x[k] = w[k];
 #pragma unroll
@@ -520,12 +541,12 @@ __device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols
 #pragma unroll
             for (int k = 0; k < h; ++k) {
                 // lanes without bit h keep value k, the others value k + h
-                const double give = up ? x[k] : x[k + h];
-                const double keep = up ? x[k + h] : x[k];
-                x[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+                const V give = up ? x[k] : x[k + h];
+                const V keep = up ? x[k + h] : x[k];
+                x[k] = keep + shfl_xor(give, h);
             }
         }
-        wv[warp * 32 + lane] = x[0];  // lane l holds value l
+        wv[warp * 32 + lane] = sum_value(x[0]);  // lane l holds value l
         __syncthreads();
         if (tid < 32) {
             double s = 0.0;
@@ -546,7 +567,7 @@ __device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols
                 if (v0 > 0 || base > 0) __syncthreads();
                 if (tid >= base && tid < base + kRedThreads) {
 #pragma unroll
-                    for (int k = 0; k < W; ++k) wv[k * kRedThreads + tid - base] = w[k];
+                    for (int k = 0; k < W; ++k) wv[k * kRedThreads + tid - base] = sum_value(w[k]);
                 }
                 __syncthreads();
                 if (adds && part < per) {
@@ -589,8 +610,8 @@ __device__ __forceinline__ void block_sums(const double (&w)[NV * RT], int ncols
 // all_frozen and the FP32 coefficients of SolverState): mixed BiCGstab on
 // 20x12x28x36 8.10 -> 5.46 ms, EigCG on 16^3x32 303 -> 272 ms (its 32-value
 // sums 234 -> 92 us), FP64 norm of a 24^3x48 half field 35 -> 25 us.
-template <int NV, int RT>
-__device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int ncols) {
+template <int NV, int RT, class V>
+__device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT, V> &acc, int ncols) {
     constexpr int W = NV * RT;
     constexpr int kWords = W == 32 ? 32 * 32 : W * kRedThreads;
     __shared__ double wv[kWords];
@@ -598,12 +619,12 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int nc
     __shared__ bool last;
     const int tid = ltid(), nthr = lsize();
     const int n = ncols * RT, slots = NV * n;
-    double w[W];
+    V first[W];
 #pragma unroll
     for (int k = 0; k < NV; ++k)
 #pragma unroll
-        for (int t = 0; t < RT; ++t) w[k * RT + t] = acc.v[k][t];
-    block_sums<NV, RT>(w, ncols, wv, slot);
+        for (int t = 0; t < RT; ++t) first[k * RT + t] = acc.v[k][t];
+    block_sums<NV, RT, V>(first, ncols, wv, slot);
     for (int t = tid; t < slots; t += nthr) red.partials[(size_t)t * kMaxReduceBlocks + blockIdx.x] = slot[t];
     __syncthreads();
     if (tid == 0) {
@@ -614,6 +635,7 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT> &acc, int nc
     __syncthreads();
     if (!last) return;
     if (ncols == 1) {
+        double w[W];
 #pragma unroll
         for (int q = 0; q < W; ++q) w[q] = 0.0;
 #pragma unroll 4
