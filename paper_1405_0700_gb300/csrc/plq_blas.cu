@@ -134,9 +134,13 @@ __global__ void dot_norm_kernel(long long N, int n, const void *av, const void *
 // p serves both updates, and q = Mhat^dagger Mhat p is never stored: per site and
 // iteration seven field accesses instead of the ten of separate x/r and p
 // updates.  24^3x48: mixed CG solve 16.7 -> 16.0 ms, FP32 x/r and p updates 31 + 14
-// -> 26 us.  x may be stored at higher precision PX.
+// -> 26 us.  x may be stored at higher precision PX.  FP64: f r also goes to the
+// FP32 slot r32 (same element order) when there is one, while it is in registers
+// (EigCG's search space on 16^3x32: 9.2 us an iteration as a pass of its own,
+// three solves 209 -> 207 ms).
 template <int P, int PX>
-__global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st) {
+__global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st, float2 *r32,
+                             double f) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
     ELEM_LOOP(N) {
@@ -162,6 +166,12 @@ __global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r
             pv[k].im = fma(beta, pv[k].im, rv[k].im);
         }
         Spinor<P>::store(p, N, e, pv);
+        if constexpr (P == PLQ_F64) {
+            if (!r32) continue;
+#pragma unroll
+            for (int k = 0; k < 12; ++k)
+                r32[(size_t)k * N + e] = make_float2((float)(f * rv[k].re), (float)(f * rv[k].im));
+        }
     }
 }
 
@@ -417,12 +427,13 @@ plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int p
     return PLQ_OK;
 }
 
-plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s) {
+plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s,
+                      float2 *r32, double f) {
     const int grid = grid_for(N, false);
     // the solution accumulator is FP64 for FP64 solves and FP32 otherwise
-    if (prec == PLQ_F64) cg_xp_kernel<PLQ_F64, PLQ_F64><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st);
-    else if (prec == PLQ_F32) cg_xp_kernel<PLQ_F32, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st);
-    else cg_xp_kernel<PLQ_F16, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st);
+    if (prec == PLQ_F64) cg_xp_kernel<PLQ_F64, PLQ_F64><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, r32, f);
+    else if (prec == PLQ_F32) cg_xp_kernel<PLQ_F32, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, nullptr, 1.0);
+    else cg_xp_kernel<PLQ_F16, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, nullptr, 1.0);
     PLQ_CUDA(cudaGetLastError());
     return PLQ_OK;
 }

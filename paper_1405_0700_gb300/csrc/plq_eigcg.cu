@@ -14,8 +14,8 @@
 // x0 = U H^{-1} U^H rhs ("init-CG").
 //
 // GPU mapping: the CG iterations are the fused kernels of the other solvers,
-// launched in batches that fill the search space; each iteration also copies
-// r_{j+1} into its slot of V, and the device records alpha_j, beta_j,
+// launched in batches that fill the search space; the pass over x and p also
+// stores r_{j+1} in its slot of V, and the device records alpha_j, beta_j,
 // |r_{j+1}|^2, from which the host builds T.  Restarts and Ritz extraction are
 // a small dense eigenproblem on the host (Jacobi, at most m = 64, some 10 ms)
 // and one linear-combination kernel over V on the device.  CG itself does not
@@ -662,12 +662,9 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, mp, to, EPI_XPAY_NORM, 0, p, -kk, FIN_CG_ALPHA, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, mp, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, r, to, EPI_XPAY_RUPD, 1, mp, -kk, FIN_CG_BETA, r, true));
-                if (eig) {  // raw r_{j+1} into its (FP32) slot of the search space
-                    to32_kernel<<<grid_of(G.N), 256, 0, s>>>(G.N, Vb + (size_t)(vs + i) * E->slot,
-                                                             static_cast<const double2 *>(r), vscale);
-                    PLQ_CUDA(cudaGetLastError());
-                }
-                return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s);
+                // the raw r_{j+1} goes into its (FP32) slot of the search space
+                return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s,
+                                  eig ? Vb + (size_t)(vs + i) * E->slot : nullptr, vscale);
             };
             for (int i = 0; i < L && st == PLQ_OK; ++i) st = body(i);
             if (st == PLQ_OK && restart) st = restart_space();

@@ -328,7 +328,8 @@ plq_status blas_norm2(long long N, int n, const void *v, int prec, const Reduce 
 plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int prec, const Reduce &red,
                          cudaStream_t s);
 // x += alpha p, then p = r + beta p unless the right-hand side has stopped; where xpend is set
-plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s);
+plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s,
+                      float2 *r32 = nullptr, double f = 1.0);
 // p = r + beta p
 plq_status blas_cg_direction(long long N, int n, void *p, const void *r, int prec, const SolverState *st,
                              cudaStream_t s);
