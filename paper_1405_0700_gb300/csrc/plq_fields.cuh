@@ -376,6 +376,8 @@ __device__ __forceinline__ void finalize_one(int fin, SolverState *state, const 
     }
     switch (fin) {
     case FIN_CG_ALPHA:
+        // an iteration that ends here (alpha not finite) updates neither x nor p
+        st->xpend = 0;
         st->pAp = tot[0];
         st->alpha = st->rho / tot[0];
         st->alpha32 = (float)st->alpha;
