@@ -139,8 +139,8 @@ __global__ void dot_norm_kernel(long long N, int n, const void *av, const void *
 // (EigCG's search space on 16^3x32: 9.2 us an iteration as a pass of its own,
 // three solves 209 -> 207 ms).
 template <int P, int PX>
-__global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st, float2 *r32,
-                             double f) {
+__global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st, LoopEnd loop,
+                             float2 *r32, double f) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
     ELEM_LOOP(N) {
@@ -173,6 +173,7 @@ __global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r
                 r32[(size_t)k * N + e] = make_float2((float)(f * rv[k].re), (float)(f * rv[k].im));
         }
     }
+    loop_end(loop, st, n);
 }
 
 // p = r + beta p
@@ -293,9 +294,11 @@ __device__ __forceinline__ cx<T> cmulc(cx<T> c, cx<T> z) {
     return {c.re * z.re - c.im * z.im, c.re * z.im + c.im * z.re};
 }
 
-// p = r + beta (p - omega v)
+// p = r + beta (p - omega v).  (The bound keeps the 32 resident warps that the call
+// in loop_end would take: 64 -> 80 registers in FP16, 128 in FP64.)
 template <int P>
-__global__ void bicg_p_kernel(long long N, int n, void *p, const void *r, const void *v, const SolverState *st) {
+__global__ void __launch_bounds__(kBlock, P == PLQ_F32 ? 5 : 4)
+bicg_p_kernel(long long N, int n, void *p, const void *r, const void *v, const SolverState *st, LoopEnd loop) {
     using T = RealOf<P>;
     ELEM_LOOP(N) {
         const int rr = rhs_of(e, n);
@@ -309,6 +312,7 @@ __global__ void bicg_p_kernel(long long N, int n, void *p, const void *r, const 
         for (int k = 0; k < 12; ++k) pv[k] = cadd(rv[k], cmulc(beta, csub(pv[k], cmulc(omega, vv[k]))));
         Spinor<P>::store(p, N, e, pv);
     }
+    loop_end(loop, st, n);
 }
 
 // s = r - alpha v
@@ -428,12 +432,12 @@ plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int p
 }
 
 plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s,
-                      float2 *r32, double f) {
+                      LoopEnd loop, float2 *r32, double f) {
     const int grid = grid_for(N, false);
     // the solution accumulator is FP64 for FP64 solves and FP32 otherwise
-    if (prec == PLQ_F64) cg_xp_kernel<PLQ_F64, PLQ_F64><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, r32, f);
-    else if (prec == PLQ_F32) cg_xp_kernel<PLQ_F32, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, nullptr, 1.0);
-    else cg_xp_kernel<PLQ_F16, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, nullptr, 1.0);
+    if (prec == PLQ_F64) cg_xp_kernel<PLQ_F64, PLQ_F64><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, r32, f);
+    else if (prec == PLQ_F32) cg_xp_kernel<PLQ_F32, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, nullptr, 1.0);
+    else cg_xp_kernel<PLQ_F16, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, nullptr, 1.0);
     PLQ_CUDA(cudaGetLastError());
     return PLQ_OK;
 }
@@ -486,9 +490,9 @@ plq_status blas_xpay64(long long N, const void *x, double a, void *y, cudaStream
 }
 
 plq_status blas_bicg_p(long long N, int n, void *p, const void *r, const void *v, int prec, const SolverState *st,
-                       cudaStream_t s) {
+                       cudaStream_t s, LoopEnd loop) {
     const int grid = grid_for(N, false);
-    DISPATCH_P(prec, bicg_p_kernel, N, n, p, r, v, st);
+    DISPATCH_P(prec, bicg_p_kernel, N, n, p, r, v, st, loop);
     PLQ_CUDA(cudaGetLastError());
     return PLQ_OK;
 }

@@ -663,7 +663,7 @@ extern "C" plq_status plq_eigcg_solve(plq_eigcg *E, void *x, const void *b, doub
                 PLQ_TRY(hop(G.S, PLQ_F64, 1, to, mp, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true));
                 PLQ_TRY(hop(G.S, PLQ_F64, 0, r, to, EPI_XPAY_RUPD, 1, mp, -kk, FIN_CG_BETA, r, true));
                 // the raw r_{j+1} goes into its (FP32) slot of the search space
-                return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s,
+                return blas_cg_xp(G.S.N, 1, xe, p, r, PLQ_F64, c->state, s, LoopEnd(),
                                   eig ? Vb + (size_t)(vs + i) * E->slot : nullptr, vscale);
             };
             for (int i = 0; i < L && st == PLQ_OK; ++i) st = body(i);

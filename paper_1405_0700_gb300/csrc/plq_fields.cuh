@@ -3,6 +3,7 @@
 #pragma once
 
 #include "plq_internal.cuh"
+#include "plq_loop.h"
 
 namespace plq {
 
@@ -512,8 +513,17 @@ __device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const 
     if (!all_frozen(st, n)) return false;
     if (red.fin == FIN_CG_ALPHA && red.st && blockIdx.x == 0)
         for (int r = ltid(); r < n; r += lsize()) red.st[r].xpend = 0;
-    if (red.cond && blockIdx.x == 0 && ltid() == 0) cudaGraphSetConditional(red.cond, 0);
     return true;
+}
+
+// The end of an iteration, in the last launch of a loop's body (the states are
+// final by then).  There and not in the finalize step: cudaGraphSetConditional is
+// a call, and a call in the reducing and the operator kernels takes registers
+// from them.
+__device__ __forceinline__ void loop_end(const LoopEnd &loop, const SolverState *st, int n) {
+    if (loop.cond == 0 || blockIdx.x != 0 || ltid() != 0) return;
+    const unsigned done = atomicAdd(loop.done, 1u) + 1;
+    if (loop_over(done, st[0].maxit, all_frozen(st, n))) cudaGraphSetConditional(loop.cond, 0);
 }
 
 // Block sums of the RedAcc values: total (value v, column c) goes to
@@ -671,10 +681,6 @@ __device__ void grid_reduce(const Reduce &red, const RedAcc<NV, RT, V> &acc, int
 #pragma unroll
             for (int k = 0; k < NV; ++k) tr[k] = slot[k * n + r];
             finalize_one(red.fin, red.st + r, tr);
-        }
-        if (red.cond) {
-            __syncthreads();
-            if (tid == 0 && all_frozen(red.st, n)) cudaGraphSetConditional(red.cond, 0);
         }
     }
     if (tid == 0) *red.ticket = 0u;

@@ -137,9 +137,12 @@ struct Reduce {
     double *sums = nullptr;       // grid totals: sums[k * nrhs + r]
     SolverState *st = nullptr;    // per right-hand side targets of the finalize step (array of nrhs)
     int fin = FIN_NONE;
-    // the loop this launch ends an iteration of (a conditional graph node): the
-    // launch ends the loop once every state has stopped; 0: no loop
+};
+
+// The device loop (conditional graph node) whose iterations a launch ends; 0: none.
+struct LoopEnd {
     unsigned long long cond = 0;
+    unsigned *done = nullptr;  // iterations of the running loop
 };
 
 constexpr int kMaxReduceBlocks = 4096;
@@ -166,7 +169,7 @@ struct Ctx {
     GaugeCopy gauge_df;  // PLQ_DF64 links (float-float, 18 reals)
     // reduction scratch
     double *partials = nullptr;         // kPartialSlots * kMaxReduceBlocks
-    unsigned *ticket = nullptr;
+    unsigned *ticket = nullptr;         // [0] the reductions', [4] LoopEnd::done, [8] the link check's
     double *sums = nullptr;             // kPartialSlots
     double *sums_host = nullptr;        // pinned mirror of sums
     SolverState *state = nullptr;       // PLQ_MAX_RHS solver states
@@ -329,7 +332,7 @@ plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int p
                          cudaStream_t s);
 // x += alpha p, then p = r + beta p unless the right-hand side has stopped; where xpend is set
 plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s,
-                      float2 *r32 = nullptr, double f = 1.0);
+                      LoopEnd loop = LoopEnd(), float2 *r32 = nullptr, double f = 1.0);
 // p = r + beta p
 plq_status blas_cg_direction(long long N, int n, void *p, const void *r, int prec, const SolverState *st,
                              cudaStream_t s);
@@ -345,7 +348,7 @@ plq_status blas_twist(long long N, void *dst, const void *src, int prec, double 
 plq_status blas_xpay64(long long N, const void *x, double a, void *y, cudaStream_t s);
 // BiCGstab: p = r + beta (p - omega v); s = r - alpha v; x += alpha p + omega s, r = s - omega t, <rhat, r>, |r|^2
 plq_status blas_bicg_p(long long N, int n, void *p, const void *r, const void *v, int prec, const SolverState *st,
-                       cudaStream_t s);
+                       cudaStream_t s, LoopEnd loop);
 plq_status blas_bicg_s(long long N, int n, void *sv, const void *r, const void *v, int prec, const SolverState *st,
                        cudaStream_t s);
 plq_status blas_bicg_update(long long N, int n, void *x, void *r, const void *p, const void *sv, const void *t,

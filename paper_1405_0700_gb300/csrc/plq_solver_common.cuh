@@ -22,7 +22,7 @@ struct Solve {
     int PX;  // inner solution accumulator precision
     double nu = 0.0;  // twisted mass: nu = 2 kappa mu (0 = Wilson)
     double hops = 0;
-    cudaGraphConditionalHandle loop = 0;  // of the loop whose body is being captured
+    LoopEnd loop;  // of the loop whose body is being captured
 };
 
 // Twisted-mass terms of one hopping launch (all zero / one for Wilson).
@@ -57,7 +57,6 @@ plq_status hop(Solve &S, int prec, int out_par, void *out, const void *in, int e
     h.lat = c->lat;
     h.red = reduce_of(c, fin);
     if (fin == FIN_NONE) h.red.st = nullptr;
-    if (fin == FIN_CG_BETA) h.red.cond = S.loop;
     h.st = freeze ? c->state : nullptr;
     h.nu_x = tw.nu_x;
     h.nu_h = tw.nu_h;
@@ -115,13 +114,13 @@ plq_status get_states(Solve &S, std::vector<SolverState> &st) {
     return PLQ_OK;
 }
 
+inline unsigned *loop_word(plq_ctx *c) { return c->ticket + 4; }
+
 // Run `body` (one inner iteration) on the device until the state of every
 // right-hand side says stop: the body is captured once into a while node of a
-// graph, whose last reduction of an iteration ends the loop.  (Every pass either
-// advances `iter` of a right-hand side that has not stopped, up to maxit, or
-// finds all stopped, so the loop ends.)  The instantiated graph is kept in
-// `cache` and reused while the key matches; the launches depend only on what
-// the key records.
+// graph, whose last launch of an iteration ends the loop (loop_end: at the latest
+// after maxit iterations).  The instantiated graph is kept in `cache` and reused
+// while the key matches; the launches depend only on what the key records.
 //
 // Batches of 16 captured iterations with a poll of the host after each ran 8
 // iterations too many per reliable-update cycle, launches that find everything
@@ -150,9 +149,9 @@ plq_status run_loop(Solve &S, Body body, std::vector<SolverState> &cur, Ctx::Sol
                                               cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             const double hops0 = S.hops;
-            S.loop = np.conditional.handle;
+            S.loop = {np.conditional.handle, loop_word(S.c)};
             for (int i = 0; i < kLoopBody && st == PLQ_OK; ++i) st = body();
-            S.loop = 0;
+            S.loop = LoopEnd();
             S.hops = hops0;
             e = cudaStreamEndCapture(S.s, &captured);
         }
@@ -165,6 +164,7 @@ plq_status run_loop(Solve &S, Body body, std::vector<SolverState> &cur, Ctx::Sol
         cache.exec = exec;
         std::memcpy(cache.key, key, sizeof(cache.key));
     }
+    PLQ_CUDA(cudaMemsetAsync(loop_word(S.c), 0, sizeof(unsigned), S.s));
     PLQ_CUDA(cudaGraphLaunch(cache.exec, S.s));
     PLQ_TRY(get_states(S, cur));
     for (int r = 0; r < S.n; ++r)

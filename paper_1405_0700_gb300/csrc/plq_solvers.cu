@@ -366,7 +366,7 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     PLQ_TRY(hop(S, PI, 1, toL, mpL, EPI_PLAIN, 1, nullptr, 0.0, FIN_NONE, nullptr, true, tw_first(S, true)));
                     // r -= alpha Mhat^dagger Mhat p, |r|^2; then x += alpha p, p = r + beta p
                     PLQ_TRY(hop(S, PI, 0, rL, toL, EPI_XPAY_RUPD, 1, mpL, -kk, FIN_CG_BETA, rL, true, tw_second(S, true)));
-                    return blas_cg_xp(S.N, n, xL, pL, rL, PI, c->state, s);
+                    return blas_cg_xp(S.N, n, xL, pL, rL, PI, c->state, s, S.loop);
                 };
                 if ((st = run_loop(S, body, fin, c->solve_graph[method], gkey)) != PLQ_OK) break;
             } else {
@@ -396,9 +396,8 @@ plq_status solve_impl(plq_ctx *c, void *x, const void *b, double kappa, int n, c
                     PLQ_TRY(hop(S, PI, 0, tL, toL, EPI_XPAY_TS, 0, sL, -kk, FIN_BICG_OMEGA, nullptr, true,
                                 tw_second(S, false)));
                     Reduce rb = reduce_of(c, FIN_BICG_RHO);
-                    rb.cond = S.loop;
                     PLQ_TRY(blas_bicg_update(S.N, n, xL, rL, pL, sL, tL, rhL, PI, rb, c->state, s));
-                    return blas_bicg_p(S.N, n, pL, rL, vL, PI, c->state, s);
+                    return blas_bicg_p(S.N, n, pL, rL, vL, PI, c->state, s, S.loop);
                 };
                 if ((st = run_loop(S, body, fin, c->solve_graph[method], gkey)) != PLQ_OK) break;
             }

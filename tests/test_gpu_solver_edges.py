@@ -9,7 +9,7 @@ from oracle import wilson as W
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_1405_0700_gb300 import F64, Context  # noqa: E402
+from paper_1405_0700_gb300 import F32, F64, Context  # noqa: E402
 from paper_1405_0700_gb300 import plq  # noqa: E402
 
 KAPPA = 0.12
@@ -83,3 +83,36 @@ def test_alpha_not_finite_leaves_the_last_iterate(solver):
         upper = U.copy()
         upper[6, ..., 1:, :, :] = 0  # (the other half of the lattice does not see these links)
         assert np.linalg.norm(other - C.wilson(upper, xs[1], KAPPA)) <= 1e-10 * np.linalg.norm(other)
+
+
+# caps around the iterations of one pass of the device loop, and below, at and above what the
+# solve needs: the loop's own bound never shows (it would be PLQ_ERR_STATE)
+@pytest.mark.parametrize("method,inner,nrhs", [("cg", F64, 1), ("cg", F32, 1), ("cg", F32, 3), ("bicgstab", F32, 1),
+                                               ("bicgstab", F64, 2)])
+def test_iteration_cap(method, inner, nrhs):
+    dims = (8, 4, 4, 4)
+    U = S.gauge_field(dims, 0.3, 51)
+    b = np.stack([S.gaussian_spinor(dims, 52 + r) for r in range(nrhs)])
+    with Context(dims) as ctx:
+        ctx.gauge_upload(U, 18, F64)
+        if inner != F64:
+            ctx.gauge_upload(U, 18, inner)
+        src = ctx.to_device(b if nrhs > 1 else b[0], F64, nrhs)
+        x = ctx.empty_full(F64, nrhs)
+
+        def solve(maxit):
+            fn = ctx.cg_solve_multi if method == "cg" else ctx.bicgstab_solve_multi
+            return fn(x, src, KAPPA, nrhs, inner_prec=inner, maxit=maxit, raise_on_error=False)
+
+        need = solve(20000)
+        assert all(i.status == plq.PLQ_OK for i in need)
+        most = max(i.iterations for i in need)
+        for maxit in [1, 2, 3, 4, 5, 6, 7, most - 1, most, most + 1]:
+            for i, full in zip(solve(maxit), need):
+                assert i.iterations <= maxit
+                if maxit >= most:
+                    assert i.status == plq.PLQ_OK and i.iterations == full.iterations
+                elif maxit <= 7:
+                    assert i.status == plq.PLQ_ERR_NOT_CONVERGED and i.iterations == maxit
+                else:  # (the residual check behind the last iteration may find it converged)
+                    assert i.status in (plq.PLQ_OK, plq.PLQ_ERR_NOT_CONVERGED)
