@@ -116,7 +116,15 @@ struct SolverState {
     // FP64 pipe.
     float alpha32, beta32;
     float2 c_alpha32, c_omega32, c_beta32;
+    // Keeps the size off a power of two (256 bytes): there the compiler turns the
+    // address of st[r].stop into shifts that it hoists, and the 80 registers of the
+    // links-in-shared-memory kernel spill 20 bytes instead of 8.  12 right-hand
+    // sides in FP32, 48^3x96 12-real 4326 -> 4209 us, 18-real 4472 -> 4349, 24^3x48
+    // 12-real 236 -> 226; 4 on 24^3x48 18-real 120 -> 111.
+    double pad[2];
 };
+
+static_assert((sizeof(SolverState) & (sizeof(SolverState) - 1)) != 0, "see SolverState::pad");
 
 enum { FLAG_NAN = 1, FLAG_BREAKDOWN = 2 };
 
