@@ -825,12 +825,16 @@ plq_status launch_mrhs_t(const HopArgs &a, cudaStream_t s, int block) {
     static std::atomic<int> per_sm[kMaxSitesPerBlock + 1][PLQ_MAX_RHS + 1];
     auto kern = hop_mrhs_kernel<P, R, EPI, DAG, RT, NB>;
     if (per_sm[spb][tiles].load(std::memory_order_relaxed) == 0) {
-        int nb = 0;
-        cudaError_t e = cudaSuccess;
-        if (smem > 48 * 1024)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int nb = 0, device = 0, optin = 0;
         cudaFuncAttributes fa{};
+        cudaGetDevice(&device);
+        cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+        // above 48 KB, the kernel's own (reducing epilogues: 2.7 KB or more) included, a
+        // block opts in: to all there is, whatever this shape takes, because the limit is
+        // the kernel's and a smaller one set for the next shape would end this one
+        if (e == cudaSuccess && fa.sharedSizeBytes + smem > 48 * 1024)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
         if (e != cudaSuccess) return cuda_error(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(hop_mrhs)");
         if (threads > fa.maxThreadsPerBlock) nb = 0;
