@@ -332,14 +332,17 @@ plq_status launch_rows_t(const HopArgs &a, cudaStream_t s) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t avail = (size_t)smem_max - 2048;  // room for the static shared memory of the kernel
+    auto kern = hop_rows_kernel<P, R, EPI, DAG>;
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return cuda_error(e, "cudaFuncGetAttributes(hop_rows_kernel)");
+    const size_t avail = (size_t)smem_max - fa.sharedSizeBytes;
     int nslot = (int)(avail / slot);
     if (a.spt > 0) nslot = a.spt < nslot ? a.spt : nslot;  // sites_per_thread selects the slot count
     if (nslot > kRowSlots) nslot = kRowSlots;
     if (nslot < 2) return set_error(PLQ_ERR_ARG, "the row-streamed kernel's slots do not fit in shared memory");
     const size_t smem = (size_t)nslot * slot;
-    auto kern = hop_rows_kernel<P, R, EPI, DAG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(hop_rows_kernel)");
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);

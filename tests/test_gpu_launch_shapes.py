@@ -54,3 +54,17 @@ def test_large_block_after_a_smaller_one():
             for r in range(12):
                 assert rel(H[r], C.hopping(U, b[r])) <= TOL[F32]
             solve_and_check(ctx, U, b)
+
+
+# rows of which 8 (300 elements) or 5 (480) fill all but 2048 bytes of a block's shared memory,
+# less than the norm epilogue needs for itself
+@pytest.mark.parametrize("lx,reals", [(50, 18), (80, 12)])
+def test_row_streamed_solve_with_full_shared_memory(lx, reals):
+    dims = (4, lx, 2, 2)
+    U = S.gauge_field(dims, 0.3, 65)
+    b = np.stack([S.gaussian_spinor(dims, 66 + r) for r in range(12)])
+    with Context(dims) as ctx:
+        ctx.gauge_upload(U, 18, F64)
+        ctx.gauge_upload(U, reals, F32)
+        ctx.set_launch(F32, 12, smem_links=4)
+        solve_and_check(ctx, U, b)
