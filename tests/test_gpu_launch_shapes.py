@@ -68,3 +68,7 @@ def test_row_streamed_solve_with_full_shared_memory(lx, reals):
         ctx.gauge_upload(U, reals, F32)
         ctx.set_launch(F32, 12, smem_links=4)
         solve_and_check(ctx, U, b)
+        for slots in (2, 3):  # slots, not sites per thread of the launches that kernel does not make
+            ctx.set_launch(F32, 12, smem_links=4, sites_per_thread=slots)
+            for method in ("cg", "bicgstab"):
+                solve_and_check(ctx, U, b, method)
