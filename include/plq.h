@@ -485,8 +485,8 @@ typedef struct {
                              (the tuner does not time it: slower on GB300);
                              5 split kernel, the eight directions of a site on eight
                              warps: the library's own choice for FP64 storage and small
-                             lattices, and a candidate of the tuner (plq_set_launch
-                             does not take it: all zeros leave the choice to the library) */
+                             lattices, and a candidate of the tuner (block 256, nothing
+                             else set: plq_set_launch takes it in this form)           */
     double us_per_launch; /* measured time of one half-lattice application                 */
     int from_cache;       /* 1 if the choice came from the cache file                      */
     int candidates;       /* configurations timed                                          */
@@ -525,10 +525,11 @@ PLQ_API plq_status plq_autotune(plq_ctx *ctx, int prec, int nrhs, const char *ca
  * (0 = library default, else a multiple of 32 up to 1024; a block the kernel
  * cannot launch makes the operator calls return PLQ_ERR_ARG), index_mode 0 or 1,
  * rhs_tile 1, 2 or 4 (dividing nrhs), z_chunk 0 or a divisor of Lz and
- * smem_links 0..4 (1..3: nrhs > 1, FP32/FP16; 4: FP32/FP16, needs nrhs x Lx/2
+ * smem_links 0..5 (1..3: nrhs > 1, FP32/FP16; 4: FP32/FP16, needs nrhs x Lx/2
  * <= 512 and, for FP16 storage, site-norm runs of 16-byte multiples, else the
- * operator calls return PLQ_ERR_ARG; with 1, rhs_tile 1 or 2; with 2, 3 or 4,
- * rhs_tile 1) and sites_per_thread 0..64, as above. */
+ * operator calls return PLQ_ERR_ARG; 5: with block 256 and all else unset; with
+ * 1, rhs_tile 1 or 2; with 2, 3 or 4, rhs_tile 1) and sites_per_thread 0..64, as
+ * above. */
 PLQ_API plq_status plq_set_launch(plq_ctx *ctx, int prec, int nrhs, int block, int index_mode, int rhs_tile,
                                   int z_chunk, int smem_links, int sites_per_thread);
 

@@ -953,22 +953,18 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
     // formats and the epilogues of operator applications and CG; the
     // neighbour-table variants for the plain and xpay epilogues; the
     // row-streamed kernel for whole-lattice applications with those epilogues.
-    if (a.smem_links == 4 && epi == EPI_XPAY_RUPD) {
-        // the row-streamed kernel has no such form: the library's choice (sites_per_thread
-        // is its number of slots and would size another kernel's grid)
+    // (the tuner times the plain form: a reducing one keeps the library's rule)
+    const bool split = a.smem_links == 5 && split_fits(a, epi) && (epi < EPI_XPAY_NORM || split_default<P>(a, epi));
+    if ((a.smem_links == 5 && !split) || (a.smem_links == 4 && epi == EPI_XPAY_RUPD)) {
+        // a split or row-streamed launch where that kernel has no such form or loses with
+        // it: the library's choice (sites_per_thread of the latter is its number of slots and would size
+        // another kernel's grid)
         HopArgs d = a;
         d.smem_links = d.block = d.spt = 0;
         d.untuned = 1;
         return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
     }
-    if (a.smem_links == 5 || a.untuned) {
-        if (split_fits(a, epi) && (a.smem_links == 5 || split_default<P>(a, epi))) return dispatch_split<P, R>(a, epi, s);
-        if (a.smem_links == 5) {  // a tuned split launch, where the split kernel has no form: the library's default
-            HopArgs d = a;
-            d.smem_links = d.block = 0;
-            return dispatch_hop<P, R>(d, epi, s, hop_default_block(P));
-        }
-    }
+    if (split || (a.untuned && split_fits(a, epi) && split_default<P>(a, epi))) return dispatch_split<P, R>(a, epi, s);
     if (a.both) {  // the parities one after the other
         HopArgs h = a;
         h.both = 0;

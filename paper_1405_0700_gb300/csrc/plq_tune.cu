@@ -29,6 +29,8 @@ __global__ void build_nbr_kernel(Lattice L, int par, int *tab) {
     }
 }
 
+constexpr int kSplitBlock = 256;  // threads of a block of the split kernel
+
 const char *prec_name(int p) { return p == PLQ_F64 ? "f64" : p == PLQ_F32 ? "f32" : "f16"; }
 
 std::string tune_key(const Ctx *c, int prec, int nrhs) {
@@ -55,7 +57,8 @@ bool cache_lookup(const char *path, const std::string &key, TuneEntry *e) {
         const int got = sscanf(line, "%599s %d %d %d %d %d %f %d", k, &block, &mode, &tile, &zc, &sm, &us, &spt);
         const bool valid = (block == 0 || (block >= 32 && block <= 1024 && block % 32 == 0)) && (mode == 0 || mode == 1) &&
                            (tile == 1 || tile == 2 || tile == 4) && zc >= 0 && sm >= 0 && sm <= 5 && spt >= 0 &&
-                           spt <= 64 && !(sm >= 2 && tile != 1) && !(sm == 1 && tile == 4);
+                           spt <= 64 && !(sm >= 2 && tile != 1) && !(sm == 1 && tile == 4) &&
+                           !(sm == 5 && (block != kSplitBlock || mode || zc || spt));
         if (got >= 7 && key == k && valid) {
             e->block = block;
             e->index_mode = mode;
@@ -237,7 +240,7 @@ extern "C" plq_status plq_autotune(plq_ctx *c, int prec, int nrhs, const char *c
     // the split kernel (its block and grid are its own)
     if (st == PLQ_OK) {
         TuneEntry t;
-        t.block = 256;
+        t.block = kSplitBlock;
         t.smem_links = 5;
         float us = -1.f;
         st = time_cfg(t, &us);
@@ -296,8 +299,10 @@ extern "C" plq_status plq_set_launch(plq_ctx *c, int prec, int nrhs, int block, 
     if (nrhs % rhs_tile) return set_error(PLQ_ERR_ARG, "rhs_tile must divide nrhs");
     if (z_chunk < 0 || (z_chunk > 0 && c->lat.L[3] % z_chunk))
         return set_error(PLQ_ERR_ARG, "z_chunk must be 0 or divide Lz");
-    if (smem_links < 0 || smem_links > 4) return set_error(PLQ_ERR_ARG, "smem_links must be 0, 1, 2, 3 or 4");
-    if (smem_links >= 2 && rhs_tile != 1) return set_error(PLQ_ERR_ARG, "smem_links 2, 3 and 4 need rhs_tile 1");
+    if (smem_links < 0 || smem_links > 5) return set_error(PLQ_ERR_ARG, "smem_links must be 0, 1, 2, 3, 4 or 5");
+    if (smem_links >= 2 && rhs_tile != 1) return set_error(PLQ_ERR_ARG, "smem_links 2 to 5 need rhs_tile 1");
+    if (smem_links == 5 && (block != kSplitBlock || index_mode || z_chunk || sites_per_thread))
+        return set_error(PLQ_ERR_ARG, "smem_links 5 goes with block %d and nothing else", kSplitBlock);
     if (smem_links == 4 && prec == PLQ_F64) return set_error(PLQ_ERR_ARG, "smem_links 4 needs FP32 or FP16 storage");
     if (smem_links == 1 && rhs_tile == 4) return set_error(PLQ_ERR_ARG, "smem_links 1 needs rhs_tile 1 or 2");
     PLQ_CUDA(cudaSetDevice(c->device));

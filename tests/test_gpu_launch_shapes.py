@@ -10,7 +10,8 @@ from oracle import c_oracle as C
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_1405_0700_gb300 import F32, F64, Context  # noqa: E402
+from paper_1405_0700_gb300 import F16, F32, F64, Context, PLQError  # noqa: E402
+from paper_1405_0700_gb300 import plq  # noqa: E402
 
 KAPPA = 0.115
 
@@ -72,3 +73,33 @@ def test_row_streamed_solve_with_full_shared_memory(lx, reals):
             ctx.set_launch(F32, 12, smem_links=4, sites_per_thread=slots)
             for method in ("cg", "bicgstab"):
                 solve_and_check(ctx, U, b, method)
+
+
+# what plq_autotune may report can be set by hand: the split kernel, in the one form it has
+@pytest.mark.parametrize("prec,nrhs", [(F64, 1), (F32, 1), (F16, 1), (F64, 3), (F32, 3), (F32, 12)])
+def test_split_launch_by_hand(prec, nrhs):
+    dims = (4, 4, 6, 4)
+    U = S.gauge_field(dims, 0.3, 67)
+    b = np.stack([S.gaussian_spinor(dims, 68 + r) for r in range(nrhs)])
+    with Context(dims) as ctx:
+        ctx.gauge_upload(U, 18, F64)
+        if prec != F64:
+            ctx.gauge_upload(U, 18, prec)
+        ctx.set_launch(prec, nrhs, 256, smem_links=5)
+        H = gpu_hopping_full(ctx, b if nrhs > 1 else b[0], prec, nrhs).reshape(b.shape)
+        for r in range(nrhs):
+            assert rel(H[r], C.hopping(U, b[r])) <= TOL[prec]
+        x = ctx.empty_full(F64, nrhs)
+        bd = ctx.to_device(b if nrhs > 1 else b[0], F64, nrhs)
+        for solve in (ctx.cg_solve_multi, ctx.bicgstab_solve_multi):  # (its reductions take one right-hand side)
+            solve(x, bd, KAPPA, nrhs, inner_prec=prec)
+            xs = ctx.to_host(x, F64, nrhs).reshape(b.shape)
+            for r in range(nrhs):
+                assert np.linalg.norm(b[r] - C.wilson(U, xs[r], KAPPA)) <= 1e-10 * np.linalg.norm(b[r])
+        tuned = ctx.autotune(prec, nrhs)
+        ctx.set_launch(prec, nrhs, *(tuned[k] for k in ("block", "index_mode", "rhs_tile", "z_chunk", "smem_links",
+                                                        "sites_per_thread")))
+        for bad in [dict(block=128), dict(index_mode=1), dict(z_chunk=2), dict(sites_per_thread=1), dict(block=0)]:
+            with pytest.raises(PLQError) as e:
+                ctx.set_launch(prec, nrhs, **dict(dict(block=256, smem_links=5), **bad))
+            assert e.value.status == plq.PLQ_ERR_ARG
