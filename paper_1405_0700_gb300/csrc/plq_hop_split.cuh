@@ -147,11 +147,18 @@ constexpr long long kSplitElements = 8192;
 // The reducing epilogues keep one right-hand side per thread: one in all.
 inline bool split_fits(const HopArgs &a, int epi) { return a.nrhs == 1 || epi <= EPI_XPAY; }
 
-// FP64 with a norm: 16^3x32 (65,536 sites) 142 us in hop_kernel, 130 here, but
-// 24^3x48 (331,776) 580 against 616 us, where blocks walk several tiles.
+// FP64 with a reduction: below the line the even spread of 32-site tiles wins, above
+// it blocks walk several tiles and hop_kernel does.  FP64 solves of 45 iterations,
+// hop_kernel / this for the reducing launches, CG and BiCGstab: 16^3x32 (65,536
+// sites) 23.75 / 22.76 and 13.90 / 13.58 ms, 16^3x40 29.21 / 27.64 and 17.35 / 16.70,
+// 16^3x48 35.18 / 33.50 and 20.36 / 19.65, 24^3x16 (110,592) 36.80 / 36.90 and 22.07 /
+// 21.36, 20^3x32 (128,000) 42.60 / 42.64 and 25.86 / 27.05, 20^3x40 53.39 / 52.75 and
+// 32.27 / 32.12, 24^3x24 (165,888) 54.79 / 55.04 and 31.69 / 33.36, 24^3x32 71.83 /
+// 72.88 and 41.05 / 41.72, 28^3x24 84.06 / 87.34 and 49.99 / 54.00 ms.
+constexpr int kSplitReduceSites = 120000;
 template <int P>
 bool split_default(const HopArgs &a, int epi) {
-    if (P == PLQ_F64) return epi < EPI_XPAY_NORM || a.lat.Vh <= 131072;
+    if (P == PLQ_F64) return epi < EPI_XPAY_NORM || a.lat.Vh <= kSplitReduceSites;
     return (long long)a.lat.Vh * a.nrhs <= kSplitElements;
 }
 
