@@ -516,14 +516,16 @@ __device__ __forceinline__ bool frozen_exit(const SolverState *st, int n, const 
     return true;
 }
 
-// The end of an iteration, in the last launch of a loop's body (the states are
-// final by then).  There and not in the finalize step: cudaGraphSetConditional is
+// The end of a pass of a loop, in its last launch (the states are final by then).  There and not in the finalize step: cudaGraphSetConditional is
 // a call, and a call in the reducing and the operator kernels takes registers
 // from them.
 __device__ __forceinline__ void loop_end(const LoopEnd &loop, const SolverState *st, int n) {
     if (loop.cond == 0 || blockIdx.x != 0 || ltid() != 0) return;
-    const unsigned done = atomicAdd(loop.done, 1u) + 1;
-    if (loop_over(done, st[0].maxit, all_frozen(st, n))) cudaGraphSetConditional(loop.cond, 0);
+    const unsigned done = atomicAdd(loop.done, loop.pass) + loop.pass;
+    if (loop_over(done, st[0].maxit, all_frozen(st, n))) {
+        *loop.done = 0;
+        cudaGraphSetConditional(loop.cond, 0);
+    }
 }
 
 // Block sums of the RedAcc values: total (value v, column c) goes to

@@ -147,10 +147,11 @@ struct Reduce {
     int fin = FIN_NONE;
 };
 
-// The device loop (conditional graph node) whose iterations a launch ends; 0: none.
+// The device loop (conditional graph node) of which a launch ends a pass; 0: none.
 struct LoopEnd {
     unsigned long long cond = 0;
-    unsigned *done = nullptr;  // iterations of the running loop
+    unsigned *done = nullptr;  // iterations of the running loop; zero before and after
+    unsigned pass = 0;         // iterations of a pass
 };
 
 constexpr int kMaxReduceBlocks = 4096;

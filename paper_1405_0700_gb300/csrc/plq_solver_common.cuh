@@ -22,7 +22,7 @@ struct Solve {
     int PX;  // inner solution accumulator precision
     double nu = 0.0;  // twisted mass: nu = 2 kappa mu (0 = Wilson)
     double hops = 0;
-    LoopEnd loop;  // of the loop whose body is being captured
+    LoopEnd loop;  // of the loop whose pass ends with the iteration being captured
 };
 
 // Twisted-mass terms of one hopping launch (all zero / one for Wilson).
@@ -118,8 +118,8 @@ inline unsigned *loop_word(plq_ctx *c) { return c->ticket + 4; }
 
 // Run `body` (one inner iteration) on the device until the state of every
 // right-hand side says stop: the body is captured once into a while node of a
-// graph, whose last launch of an iteration ends the loop (loop_end: at the latest
-// after maxit iterations).  The instantiated graph is kept in `cache` and reused
+// graph, whose last launch ends the loop (loop_end: at the latest once maxit
+// iterations are done).  The instantiated graph is kept in `cache` and reused
 // while the key matches; the launches depend only on what the key records.
 //
 // Batches of 16 captured iterations with a poll of the host after each ran 8
@@ -149,8 +149,10 @@ plq_status run_loop(Solve &S, Body body, std::vector<SolverState> &cur, Ctx::Sol
                                               cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             const double hops0 = S.hops;
-            S.loop = {np.conditional.handle, loop_word(S.c)};
-            for (int i = 0; i < kLoopBody && st == PLQ_OK; ++i) st = body();
+            for (int i = 0; i < kLoopBody && st == PLQ_OK; ++i) {
+                if (i == kLoopBody - 1) S.loop = {np.conditional.handle, loop_word(S.c), kLoopBody};
+                st = body();
+            }
             S.loop = LoopEnd();
             S.hops = hops0;
             e = cudaStreamEndCapture(S.s, &captured);
@@ -164,7 +166,6 @@ plq_status run_loop(Solve &S, Body body, std::vector<SolverState> &cur, Ctx::Sol
         cache.exec = exec;
         std::memcpy(cache.key, key, sizeof(cache.key));
     }
-    PLQ_CUDA(cudaMemsetAsync(loop_word(S.c), 0, sizeof(unsigned), S.s));
     PLQ_CUDA(cudaGraphLaunch(cache.exec, S.s));
     PLQ_TRY(get_states(S, cur));
     for (int r = 0; r < S.n; ++r)
