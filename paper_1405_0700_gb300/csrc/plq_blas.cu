@@ -138,9 +138,13 @@ __global__ void dot_norm_kernel(long long N, int n, const void *av, const void *
 // FP32 slot r32 (same element order) when there is one, while it is in registers
 // (EigCG's search space on 16^3x32: 9.2 us an iteration as a pass of its own,
 // three solves 209 -> 207 ms).
-template <int P, int PX>
-__global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st, LoopEnd loop,
-                             float2 *r32, double f) {
+// LOOP: the launch ends a pass of the device loop.  The call in loop_end takes
+// registers (FP32 112 -> 136, one resident block fewer: mixed CG on 24^3x48 15.77 ->
+// 16.12 ms), so it is in this form only, and bounded.
+template <int P, int PX, bool LOOP>
+__global__ void __launch_bounds__(kBlock, LOOP && P != PLQ_F64 ? 2 : 0)
+cg_xp_kernel(long long N, int n, void *x, void *p, const void *r, const SolverState *st, LoopEnd loop, float2 *r32,
+             double f) {
     using T = RealOf<P>;
     using TX = RealOf<PX>;
     ELEM_LOOP(N) {
@@ -173,7 +177,7 @@ __global__ void cg_xp_kernel(long long N, int n, void *x, void *p, const void *r
                 r32[(size_t)k * N + e] = make_float2((float)(f * rv[k].re), (float)(f * rv[k].im));
         }
     }
-    loop_end(loop, st, n);
+    if constexpr (LOOP) loop_end(loop, st, n);
 }
 
 // p = r + beta p
@@ -294,10 +298,9 @@ __device__ __forceinline__ cx<T> cmulc(cx<T> c, cx<T> z) {
     return {c.re * z.re - c.im * z.im, c.re * z.im + c.im * z.re};
 }
 
-// p = r + beta (p - omega v).  (The bound keeps the 32 resident warps that the call
-// in loop_end would take: 64 -> 80 registers in FP16, 128 in FP64.)
-template <int P>
-__global__ void __launch_bounds__(kBlock, P == PLQ_F32 ? 5 : 4)
+// p = r + beta (p - omega v).  LOOP as above (64 -> 80 registers in FP16, 128 in FP64).
+template <int P, bool LOOP>
+__global__ void __launch_bounds__(kBlock, P == PLQ_F64 ? 4 : !LOOP ? 0 : P == PLQ_F32 ? 5 : 4)
 bicg_p_kernel(long long N, int n, void *p, const void *r, const void *v, const SolverState *st, LoopEnd loop) {
     using T = RealOf<P>;
     ELEM_LOOP(N) {
@@ -312,7 +315,7 @@ bicg_p_kernel(long long N, int n, void *p, const void *r, const void *v, const S
         for (int k = 0; k < 12; ++k) pv[k] = cadd(rv[k], cmulc(beta, csub(pv[k], cmulc(omega, vv[k]))));
         Spinor<P>::store(p, N, e, pv);
     }
-    loop_end(loop, st, n);
+    if constexpr (LOOP) loop_end(loop, st, n);
 }
 
 // s = r - alpha v
@@ -434,10 +437,12 @@ plq_status blas_dot_norm(long long N, int n, const void *a, const void *b, int p
 plq_status blas_cg_xp(long long N, int n, void *x, void *p, const void *r, int prec, const SolverState *st, cudaStream_t s,
                       LoopEnd loop, float2 *r32, double f) {
     const int grid = grid_for(N, false);
+    const bool end = loop.cond != 0;
     // the solution accumulator is FP64 for FP64 solves and FP32 otherwise
-    if (prec == PLQ_F64) cg_xp_kernel<PLQ_F64, PLQ_F64><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, r32, f);
-    else if (prec == PLQ_F32) cg_xp_kernel<PLQ_F32, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, nullptr, 1.0);
-    else cg_xp_kernel<PLQ_F16, PLQ_F32><<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, nullptr, 1.0);
+    auto kern = prec == PLQ_F64   ? (end ? cg_xp_kernel<PLQ_F64, PLQ_F64, true> : cg_xp_kernel<PLQ_F64, PLQ_F64, false>)
+                : prec == PLQ_F32 ? (end ? cg_xp_kernel<PLQ_F32, PLQ_F32, true> : cg_xp_kernel<PLQ_F32, PLQ_F32, false>)
+                                  : (end ? cg_xp_kernel<PLQ_F16, PLQ_F32, true> : cg_xp_kernel<PLQ_F16, PLQ_F32, false>);
+    kern<<<grid, kBlock, 0, s>>>(N, n, x, p, r, st, loop, prec == PLQ_F64 ? r32 : nullptr, f);
     PLQ_CUDA(cudaGetLastError());
     return PLQ_OK;
 }
@@ -492,7 +497,11 @@ plq_status blas_xpay64(long long N, const void *x, double a, void *y, cudaStream
 plq_status blas_bicg_p(long long N, int n, void *p, const void *r, const void *v, int prec, const SolverState *st,
                        cudaStream_t s, LoopEnd loop) {
     const int grid = grid_for(N, false);
-    DISPATCH_P(prec, bicg_p_kernel, N, n, p, r, v, st, loop);
+    const bool end = loop.cond != 0;
+    auto kern = prec == PLQ_F64   ? (end ? bicg_p_kernel<PLQ_F64, true> : bicg_p_kernel<PLQ_F64, false>)
+                : prec == PLQ_F32 ? (end ? bicg_p_kernel<PLQ_F32, true> : bicg_p_kernel<PLQ_F32, false>)
+                                  : (end ? bicg_p_kernel<PLQ_F16, true> : bicg_p_kernel<PLQ_F16, false>);
+    kern<<<grid, kBlock, 0, s>>>(N, n, p, r, v, st, loop);
     PLQ_CUDA(cudaGetLastError());
     return PLQ_OK;
 }
