@@ -51,13 +51,16 @@ __device__ __forceinline__ cx<R> mul_ipow(cx<R> z) {
 
 // ---------------------------------------------------------------- launches
 // Kernels of a chain begin with chain_begin() and are launched by
-// launch_chained (programmatic dependent launch): the next kernel's blocks come
-// onto the SMs as soon as this one's have all started and leave room, and wait
-// there for its completion, instead of being launched after it.
-__device__ __forceinline__ void chain_begin() {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
+// launch_chained (programmatic dependent launch): the next kernel's blocks start
+// once this one's have all left, and wait for its memory, instead of being launched
+// after it.  No kernel lets its dependents go earlier (griddepcontrol.
+// launch_dependents): with that at the start of a kernel, the third kernel of a
+// chain could be resident while the first still ran, and read-only loads (__ldg)
+// are not kept coherent over a kernel's life; the waiting blocks also took the SMs
+// unevenly (FP64 plq_schur_apply, 8^4 48.5 -> 19.9 us without, 16x8^2x16 51.3 ->
+// 35.6; FP32 16^4 12-real 16.6 -> 11.7, 24^3x48 67.7 -> 65.2 us; with it behind the
+// last site instead: 24^3x48 74.0 us).
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 template <class... P, class... A>
 cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t s, A &&...args) {

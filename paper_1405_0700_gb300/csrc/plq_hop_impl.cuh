@@ -38,12 +38,13 @@ __device__ __forceinline__ void twist12(cx<T> v[12], T nu, T scale) {
 }
 
 // Whether a one-RHS launch is chained (launch_chained): operator calls in FP32
-// and FP64.  One after the other, hop_kernel -> chained: FP32 18-real 32^3x64 121.3
-// -> 119.1 us, 24^3x48 37.3 -> 34.9 us, plq_schur_apply on 24^3x48 86.6 -> 83.0 and
-// on 16^4 16.6 -> 12.8-14.2 us, FP64 on 16^4 119.4 -> 114.1 us.  The iterations of
-// the solvers, captured in graphs, lost (mixed CG on 24^3x48 15.87 -> 16.12 ms), and
-// so did several right-hand sides (3: 76.3 -> 77.7 us) and FP16 storage
-// (plq_schur_apply on 24^3x48 56.3 -> 59.3 us); they run unchained.
+// and FP64.  One after the other, unchained -> chained: FP32 18-real 32^3x64 120.8
+// -> 117.5 us, 24^3x48 37.2 -> 34.7 us, plq_schur_apply on 24^3x48 86.3 -> 80.5 and
+// on 16^4 16.6 -> 11.7 us, FP64 on 16^4 118.8 -> 113.5 us.  With dependents let go at
+// the start of a kernel, the iterations of the solvers, captured in graphs, lost
+// (mixed CG on 24^3x48 15.87 -> 16.12 ms), and so did several right-hand sides (3:
+// 76.3 -> 77.7 us) and FP16 storage (plq_schur_apply on 24^3x48 56.3 -> 59.3 us); they
+// run unchained.
 template <int P>
 __host__ __device__ __forceinline__ bool chained(const HopArgs &a) {
     return P != PLQ_F16 && a.st == nullptr && a.nrhs == 1;

@@ -14,8 +14,8 @@
 // site here -- the signs of the reconstruction are those of additions -- and
 // blocks of 32 sites spread them evenly where the 128-thread blocks of a one-wave
 // grid leave a nearly empty second wave.  Two applications (plq_schur_apply),
-// hop_kernel -> this: FP64 8^4 71 -> 25 us, 12^3x16 70 -> 56, 16^3x32 253 -> 226,
-// 24^3x32 745 -> 725, 24^3x48 1110 -> 1079 us; one application 32^3x64 1628 ->
+// hop_kernel -> this: FP64 8^4 71 -> 25 us (chained 20), 12^3x16 70 -> 56 (51), 16^3x32
+// 253 -> 226 (222), 24^3x32 745 -> 725 (719), 24^3x48 1110 -> 1079 us; one application 32^3x64 1628 ->
 // 1619 us, 24^3x48 with 12 right-hand sides 6167 -> 6132 us; both parities in one
 // launch (plq_wilson_apply) 16^3x32 236 -> 217 us.  Three blocks per SM
 // with a few spilled registers beat two without (16^3x32 230, 24^3x48 1102 us).
