@@ -948,6 +948,12 @@ plq_status dispatch_tiled(const HopArgs &a, int epi, cudaStream_t s, int block) 
 
 namespace plq {
 
+// The multi-RHS kernel has the epilogues of operator applications and CG, on whole
+// lattices; other launches keep hop_kernel and its default block.
+inline bool staged_form(const HopArgs &a, int epi) {
+    return a.nrhs > 1 && a.site_begin == 0 && a.site_end < 0 && (epi <= EPI_XPAY_NORM || epi == EPI_XPAY_RUPD);
+}
+
 template <int P, int R>
 plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
     // Right-hand-side tiles (RT > 1) exist for the FP32-arithmetic storage
@@ -980,13 +986,15 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
     if constexpr (P != PLQ_F64) {
         // Links staged in shared memory or read by every right-hand side's thread:
         // staging costs two barriers per block and pays once enough right-hand sides
-        // share a link.  FP32, direct / staged (blocks of 96): 24^3x48 12-real 9 RHS
-        // 206 / 222 us, 11 RHS 259 / 249, 12 RHS 274 / 236; 32^3x64 10 RHS 792 / 810,
-        // 11 RHS 898 / 830; 48^3x96 12 RHS 5683 / 4306, 18-real 5277 / 4457 (32^3x64
-        // 18-real 12 RHS 842 / 865 is the exception).  FP16, direct / staged (128):
-        // 24^3x48 12-real 3 RHS 76 / 78, 5 RHS 122 / 115, 9 RHS 219 / 191, 12 RHS
-        // 317 / 247; 32^3x64 18-real 5 RHS 375 / 379, 9 RHS 677 / 642.
-        if (a.untuned && a.nrhs >= (P == PLQ_F16 ? 5 : 11)) {
+        // share a link.  FP32, direct / staged (blocks of 96), us: 24^3x48 12-real 9 RHS
+        // 206 / 222, 11 RHS 258 / 230, 12 RHS 276 / 225; 32^3x64 10 RHS 792 / 810, 18-real
+        // 11 RHS 918 / 861, 12 RHS 860 / 877 (the exception), 12-real 905 / 843; 48^3x96
+        // 12 RHS 5576 / 4209, 18-real 5289 / 4349.  FP16 (blocks of 128) 12-real: 24^3x48
+        // 4 RHS 98 / 93, 5 RHS 121 / 115, 9 RHS 218 / 196; 32^3x64 4 RHS 298 / 303, 5 RHS
+        // 381 / 375; 18-real: 24^3x48 5 RHS 117 / 120, 6 RHS 142 / 135; 32^3x64 5 RHS 364 /
+        // 388, 6 RHS 438 / 425, 8 RHS 562 / 567, 9 RHS 655 / 651.
+        const int least = P == PLQ_F32 ? 11 : R == 12 ? 5 : 6;
+        if (a.untuned && a.nrhs >= least && staged_form(a, epi)) {
             HopArgs d = a;
             d.untuned = 0;
             d.smem_links = 1;
@@ -999,7 +1007,7 @@ plq_status dispatch_hop(const HopArgs &a, int epi, cudaStream_t s, int block) {
         const bool cg_epi = epi <= EPI_XPAY_NORM || epi == EPI_XPAY_RUPD;
         if (a.smem_links == 4 && a.site_begin == 0 && a.site_end < 0 && epi <= EPI_XPAY_NORM)
             return dispatch_rows<P, R>(a, epi, s);
-        if (a.smem_links && a.nrhs > 1 && a.site_begin == 0 && a.site_end < 0 && cg_epi) {
+        if (a.smem_links && staged_form(a, epi)) {
             if (a.rhs_tile == 2 && a.nrhs % 2 == 0) return dispatch_mrhs<P, R, 2, 0>(a, epi, s, block);
             if (a.smem_links == 2) return dispatch_mrhs<P, R, 1, 2>(a, epi, s, block);
             if (a.smem_links == 3) return dispatch_mrhs<P, R, 1, 3>(a, epi, s, block);
