@@ -508,8 +508,8 @@ typedef struct {
  * copied ahead asynchronously, the GPU counterpart of the paper's software
  * prefetch, Sec. 2.2), and with the sites walked in z-chunks of 8 or 4 planes (time
  * inside a chunk, which keeps the data reused through the time direction
- * within L2 for large multi-RHS fields), then the fastest of these with 1, 2,
- * 4 or 8 sites per thread against its one-wave grid, and keeps the fastest in
+ * within L2 for large multi-RHS fields), then the fastest few of these with 1, 2,
+ * 4 or 8 sites per thread against their one-wave grids, and keeps the fastest in
  * the context for every later operator and solver call of that precision.
  * cache_path (NULL: the PLQ_TUNE_CACHE environment variable, if set) names a
  * text file keyed by GPU name, lattice, precision, link format and nrhs: a

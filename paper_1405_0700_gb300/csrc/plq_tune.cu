@@ -3,6 +3,7 @@
 // neighbour table that plays the role of the pointer arrays of Sec. 2.2).
 // Results are kept per (precision, nrhs) in the context and, optionally, in a
 // text cache keyed by GPU name, lattice, precision, link format and nrhs.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -166,8 +167,11 @@ extern "C" plq_status plq_autotune(plq_ctx *c, int prec, int nrhs, const char *c
     struct Cand {
         int mode, tile, zc, smem;
     };
-    Cand cands[32];
+    constexpr int kCands = 32, kBlocks = sizeof blocks / sizeof blocks[0];
+    Cand cands[kCands];
     int nc = 0;
+    TuneEntry timed[kCands * kBlocks + 1];  // what could be launched, with its time
+    int nt = 0;
     const int Lz = c->lat.L[3];
     int zcs[3] = {0, 0, 0}, nz = 1;
     for (int z : {8, 4})
@@ -231,9 +235,9 @@ extern "C" plq_status plq_autotune(plq_ctx *c, int prec, int nrhs, const char *c
             float us = -1.f;
             st = time_cfg(t, &us);
             if (st != PLQ_OK) break;
-            if (us >= 0.f && us < best.us) {
+            if (us >= 0.f) {
                 t.us = us;
-                best = t;
+                timed[nt++] = t;
             }
         }
     }
@@ -244,22 +248,30 @@ extern "C" plq_status plq_autotune(plq_ctx *c, int prec, int nrhs, const char *c
         t.smem_links = 5;
         float us = -1.f;
         st = time_cfg(t, &us);
-        if (st == PLQ_OK && us >= 0.f && us < best.us) {
+        if (st == PLQ_OK && us >= 0.f) {
             t.us = us;
-            best = t;
+            timed[nt++] = t;
         }
     }
-    // sites per thread: a grid sized for k sites (site blocks) per thread
-    // against the one-wave grid of the sweep above
-    for (int k : {1, 2, 4, 8}) {
-        if (st != PLQ_OK || best.smem_links == 5) break;
-        TuneEntry t = best;
-        t.spt = k;
-        float us = -1.f;
-        st = time_cfg(t, &us);
-        if (st == PLQ_OK && us >= 0.f && us < best.us) {
-            t.us = us;
-            best = t;
+    // sites per thread: a grid sized for k sites (site blocks) per thread against the
+    // one-wave grid of the sweep above, for the best of that sweep and not its winner
+    // alone: one wave hides what the shapes differ in (FP16 12-real, 12 right-hand
+    // sides on 48^3x96: blocks of 96 to 1024 threads within a percent of each other,
+    // with 8 sites per thread 3.48 to 3.81 ms; FP32 18-real on 32^3x64 863 -> 772 us)
+    std::sort(timed, timed + nt, [](const TuneEntry &x, const TuneEntry &y) { return x.us < y.us; });
+    if (nt > 0) best = timed[0];
+    for (int q = 0; q < nt && q < (nrhs > 1 ? 16 : 4) && timed[q].us <= 1.08f * timed[0].us; ++q) {
+        if (timed[q].smem_links == 5) continue;
+        for (int k : {1, 2, 4, 8}) {
+            if (st != PLQ_OK) break;
+            TuneEntry t = timed[q];
+            t.spt = k;
+            float us = -1.f;
+            st = time_cfg(t, &us);
+            if (st == PLQ_OK && us >= 0.f && us < best.us) {
+                t.us = us;
+                best = t;
+            }
         }
     }
     cudaEventDestroy(e0);
