@@ -229,8 +229,10 @@ __global__ void zlincomb32_kernel(long long N, const float2 *in, size_t stride, 
 }
 
 // What one element adds to (re, im) of <a, b>.  FP64: two fused multiply-adds a
-// component.  FP32: the sums stay exact to ~2^-47 (SumFF) and take the rounding
-// error of one of the two products along.
+// component.  FP32: each term is rounded to FP32 once (the fused multiply-add; the
+// other product's rounding error goes along), the terms are added to ~2^-47 (SumFF).
+// Against FP64 sums of terms rounded twice: rms error of <a, b> over 16^3x32, random
+// a and b of norm one, 3.0e-11 instead of 4.9e-11.
 __device__ __forceinline__ void dot_add(double &re, double &im, double2 a, double2 b) {
     re = fma(a.x, b.x, fma(a.y, b.y, re));
     im = fma(a.x, b.y, fma(-a.y, b.x, im));

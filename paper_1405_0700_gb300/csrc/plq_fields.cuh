@@ -221,7 +221,7 @@ struct Spinor<PLQ_F16> {
         for (int k = 0; k < 3; ++k) __stcs(p + k * stride, halves(v + 4 * k, inv));
         __stcs(reinterpret_cast<float *>(static_cast<uint4 *>(base) + 3 * stride) + e, m);
     }
-    // The same store written out.  The compiler schedules hop_kernel differently
+    // The same store written out.  The compiler (nvcc 13.0) schedules hop_kernel differently
     // around the two forms: 18-real links are faster with this one (32^3x64 77.1
     // against 79.7 us, plq_wilson_apply on 24^3x48 54.2 against 62.1 us), 12-real
     // ones with the other (83.9 against 76.7 us) but for the xpay epilogue
@@ -487,19 +487,6 @@ __device__ __forceinline__ void red_init(RedAcc<NV, RT> &acc) {
     for (int k = 0; k < NV; ++k)
 #pragma unroll
         for (int t = 0; t < RT; ++t) acc.v[k][t] = 0.0;
-}
-
-// Sum over the lanes of a warp that may be partial (the block's thread count
-// need not be a multiple of 32); lane 0 gets the total.
-template <class V>
-__device__ __forceinline__ V warp_sum(V x, int lane, int active) {
-    const unsigned mask = active >= 32 ? 0xffffffffu : ((1u << active) - 1u);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const V y = __shfl_down_sync(mask, x, o);
-        if (lane + o < active) x += y;
-    }
-    return x;
 }
 
 // Every one of n right-hand sides frozen.  A reducing kernel may then leave at

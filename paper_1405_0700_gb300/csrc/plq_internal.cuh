@@ -140,7 +140,7 @@ enum Finalize {
 };
 
 struct Reduce {
-    double *partials = nullptr;   // kPartialSlots doubles per block
+    double *partials = nullptr;   // block b's sum of slot t at [t * kMaxReduceBlocks + b]
     unsigned *ticket = nullptr;   // zero on entry, left zero on exit
     double *sums = nullptr;       // grid totals: sums[k * nrhs + r]
     SolverState *st = nullptr;    // per right-hand side targets of the finalize step (array of nrhs)
