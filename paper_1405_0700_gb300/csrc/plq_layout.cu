@@ -40,10 +40,9 @@ __device__ __forceinline__ int pair_odd(const Lattice &L, int i) {
 //
 // Packing reads the records, and reads of a record's pieces one after the other
 // hit L1, so the direct form (pack_direct_kernel) stays the faster one except
-// for FP64 storage with several right-hand sides: FP64 1 / 3 / 12 RHS 48 / 141 /
-// 542 us direct against 60 / 122 / 457 us, FP16 35 / 98 / 383 against 56 / 107 /
-// 400 us; on 28x22x14x6 FP64 with 3 RHS 10.9 against 12.9 us, with 12 43.8
-// against 41.5 us.  See pack_staged().
+// for FP64 storage with some counts of right-hand sides (pack_staged): FP64 1 / 3 RHS 48 /
+// 141 us direct against 60 / 122 us on 24^3x48, FP16 1 / 3 / 12 RHS 35 / 98 / 383 against 56 /
+// 107 / 400 us; on 28x22x14x6 FP64 with 3 RHS 10.9 against 12.9 us.
 //
 // In shared memory a site record takes 13 slots of 16 bytes and a right-hand
 // side 2S * 13 + 1: both odd, so neighbouring sites and right-hand sides fall
@@ -59,7 +58,14 @@ int layout_pairs(int nrhs) {
     return S;
 }
 
-bool pack_staged(int prec, int nrhs) { return prec == PLQ_F64 && nrhs >= 4; }
+// Where two thirds of the block's threads hold an element in the packing phase (6, 11
+// and 12 right-hand sides).  Direct / staged, 4 to 12 RHS on 16^3x32: 37.0 / 46.8, 47.2 /
+// 57.5, 58.6 / 49.8, 67.2 / 80.1, 72.8 / 86.5, 78.9 / 100.3, 93.7 / 107.6, 105.9 / 86.3,
+// 112.9 / 94.1 us; on 32^3x64 6 RHS 873 / 710, 8 RHS 1157 / 1293, 11 RHS 1612 / 1287, 12 RHS
+// 1746 / 1414 us; on 28x22x14x6 6 RHS 20.4 / 19.6, 11 RHS 39.8 / 39.0 us.
+bool pack_staged(int prec, int nrhs) {
+    return prec == PLQ_F64 && nrhs >= 4 && 3 * 2 * layout_pairs(nrhs) * nrhs >= 2 * kLayoutThreads;
+}
 
 template <int P>
 __global__ void pack_direct_kernel(Lattice L, int nrhs, char *out, const double *in, size_t half_bytes) {
